@@ -1,149 +1,588 @@
 // FP64 dense kernels of the prefactorisation (Sec. 7.2: Eq. cms_boundary
 // and the reduced system of Eq. global_subspace / Eq. dd, computed on the
-// device): batched blocked Cholesky, inverse of an SPD matrix from its
-// factor, and a batched FP64 GEMM.  Row-major storage throughout; matrices
-// handed to the blocked routines are padded to a multiple of the 64-wide
-// block with identity rows/columns.
+// device): the batched inverse of SPD matrices and a batched GEMM, row-major
+// storage.  Matrices handed to the inverse are padded to a multiple of the
+// 64-wide block with identity rows/columns.
+//
+// This chip issues two FP64 FMAs per clock and SM (1.2 TFLOP/s in all): one
+// 64 x 64 x 64 product on one SM took 82 us.  So the products run on the
+// BF16 tensor cores without giving up FP64: the error-free splitting of
+// Ozaki, Ogita, Oishi and Rump ("Error-free transformations of matrix
+// multiplication", 2012) in fixed point.  Per row of 64 values, a common
+// power of two makes every value a 62-bit integer, cut into eight balanced
+// base-256 digits (-128 .. 127, exact in BF16).  A product of two digits has
+// at most 14 bits, so the FP32 accumulators hold the sums over 64 values of
+// all pairs (i, j) of one order i + j = d exactly (at most 8 x 64 x 2^14 =
+// 2^23).  The orders 0 .. 7 (36 pairs) are combined in 64-bit integers and
+// rounded once; the dropped orders are below 2^-60 of the row maxima's
+// product (FP64's own rounding is 2^-53).  Rows with an infinity or a NaN
+// give NaN.
+#include <algorithm>
+
 #include "pd_internal.h"
 
 namespace pdg {
 
 namespace {
 
-constexpr int NB = 64;   // diagonal block size of the blocked algorithms
+constexpr int NB = 64;        // block of the inverse, tile of the GEMM
+constexpr int kDig = 8;       // digits of a value
+constexpr int kThr = 512;     // threads of the digit kernels: 16 warps, one 16 x 16 part of a 64 x 64 tile each
+// digits of one 64 x 64 block: [16-column group 4][16-row group 4][digit 8]
+// fragments of 32 lanes x 16 bytes, in the register order of the A operand
+// of mma.m16n8k16 (which, for the transposed operand, is also the order of
+// two neighbouring B operands); 16 KB per 16-column group
+constexpr int kGrpVec = 4 * kDig * 32;
+constexpr int kBlkVec = 4 * kGrpVec;
+constexpr int kNanExp = 1 << 28;   // exponent of a row that holds an infinity or a NaN
+constexpr int kSmemDig = 2 * 16 * kBlkVec;   // dynamic shared memory: the digits of two blocks (128 KB)
 
-// C = alpha op(A) op(B) + beta C, 64x64 tile per block, k-step 16, 4x4 outputs per
-// thread (rows ty + 16 i, columns tx + 16 j).  lower_only: skip tiles above the
-// diagonal and write only entries with row >= column.
-__global__ void __launch_bounds__(256) k_dgemm(int M, int N, int K, double alpha, const double* __restrict__ A,
-                                               int lda, int64_t sA, int ta, const double* __restrict__ B, int ldb,
-                                               int64_t sB, int tb, double beta, double* __restrict__ C, int ldc,
-                                               int64_t sC, int lower_only) {
-    const int row0 = blockIdx.y * 64, col0 = blockIdx.x * 64;
-    if (lower_only && row0 + 63 < col0) return;
-    A += (int64_t)blockIdx.z * sA;
-    B += (int64_t)blockIdx.z * sB;
-    C += (int64_t)blockIdx.z * sC;
-    __shared__ double As[16][65];
-    __shared__ double Bs[16][65];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    double acc[4][4];
+// Exponent field -> E with |x| < 2^E for every x of that or a smaller field.
+__device__ __forceinline__ int row_exponent(int field) {
+    return field == 2047 ? kNanExp : (field == 0 ? 0 : field - 1022);
+}
+
+__device__ __forceinline__ int exponent_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// round(x 2^(62 - E)) plus the bias that makes bytes 0..6 balanced digits (|x| < 2^E; subnormals count as 0)
+__device__ __forceinline__ long long biased_fixed(double x, int E) {
+    constexpr long long kBias = 0x80808080808080ll;
+    const long long bits = __double_as_longlong(x);
+    const int ex = (int)((bits >> 52) & 0x7ff);
+    if (ex == 0 || E == kNanExp) return kBias;
+    const long long m = (bits & 0xfffffffffffffll) | (1ll << 52);
+    const int sh = ex - 1013 - E;   // <= 9
+    const long long v = sh >= 0 ? m << sh : (sh > -54 ? (m + (1ll << (-sh - 1))) >> -sh : 0);
+    return (bits < 0 ? -v : v) + kBias;
+}
+
+// digit d (0 = most significant) of a biased value, as the bits of a float
+__device__ __forceinline__ uint32_t digit_bits(long long u, int d) {
+    if (d == 0) return __float_as_uint((float)(int)(u >> 56));
+    const uint32_t byte = (uint32_t)(u >> (8 * (7 - d))) & 0xffu;
+    return __float_as_uint(__uint_as_float(0x4b000000u | byte) - 8388736.0f);
+}
+
+// x 2^n (by the exponent field where the result is a normal number)
+__device__ __forceinline__ double scale2(double x, int n) {
+    const int f = exponent_field(x);
+    if (f == 0 || f + n <= 0 || f + n >= 2047) return f == 0 ? 0.0 : ldexp(x, n);
+    return __hiloint2double(__double2hiint(x) + (n << 20), __double2loint(x));
+}
+
+// Digits of the 16 x 16 block (mb, k16) of sm, whose rows have exponents es: one fragment per digit.
+__device__ __forceinline__ void digits_block(const double (*sm)[NB + 1], const int* es, int mb, int k16, int lane,
+                                             uint4* dst) {
+    const int r = 16 * mb + (lane >> 2), c = 16 * k16 + 2 * (lane & 3);
+    const int e0 = es[r], e1 = es[r + 8];
+    const long long u0 = biased_fixed(sm[r][c], e0), u1 = biased_fixed(sm[r][c + 1], e0);
+    const long long u2 = biased_fixed(sm[r + 8][c], e1), u3 = biased_fixed(sm[r + 8][c + 1], e1);
+    const long long u4 = biased_fixed(sm[r][c + 8], e0), u5 = biased_fixed(sm[r][c + 9], e0);
+    const long long u6 = biased_fixed(sm[r + 8][c + 8], e1), u7 = biased_fixed(sm[r + 8][c + 9], e1);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int d = 0; d < kDig; ++d)   // two exact BF16 values: the upper halves of two floats
+        dst[d * 32 + lane] = make_uint4(__byte_perm(digit_bits(u0, d), digit_bits(u1, d), 0x7632),
+                                        __byte_perm(digit_bits(u2, d), digit_bits(u3, d), 0x7632),
+                                        __byte_perm(digit_bits(u4, d), digit_bits(u5, d), 0x7632),
+                                        __byte_perm(digit_bits(u6, d), digit_bits(u7, d), 0x7632));
+}
+
+// Row exponents (es: 64 ints of shared memory) and digits of the 64 x 64 block in sm.  Synchronises once; the
+// digits are complete after the caller's next barrier.
+__device__ __noinline__ void split_block(const double (*sm)[NB + 1], int* es, uint4* dig) {
+    const int r = threadIdx.x >> 3;
+    int f = 0;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        for (int l = threadIdx.x; l < 1024; l += 256) {
-            int i, k;
-            if (!ta) { i = l / 16; k = l % 16; } else { k = l / 64; i = l % 64; }
-            const int gi = row0 + i, gk = k0 + k;
-            double v = 0.0;
-            if (gi < M && gk < K) v = ta ? A[(int64_t)gk * lda + gi] : A[(int64_t)gi * lda + gk];
-            As[k][i] = v;
+    for (int k = 0; k < 8; ++k) f = max(f, exponent_field(sm[r][(threadIdx.x & 7) + 8 * k]));
+    f = max(f, __shfl_xor_sync(0xffffffffu, f, 1));
+    f = max(f, __shfl_xor_sync(0xffffffffu, f, 2));
+    f = max(f, __shfl_xor_sync(0xffffffffu, f, 4));
+    if ((threadIdx.x & 7) == 0) es[r] = row_exponent(f);
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, mb = warp >> 2, k16 = warp & 3;
+    digits_block(sm, es, mb, k16, threadIdx.x & 31, dig + (k16 * 4 + mb) * kDig * 32);
+}
+
+// A block's digits from shared to global memory (after a barrier).
+__device__ __forceinline__ void store_digits(uint4* dst, const uint4* src, int* ex, const int* es) {
+    for (int l = threadIdx.x; l < kBlkVec; l += kThr) dst[l] = src[l];
+    if (threadIdx.x < NB) ex[threadIdx.x] = es[threadIdx.x];
+}
+
+// The digits of two blocks from global to shared memory, one group of asynchronous copies per 16 columns.
+__device__ __forceinline__ void load_digits(uint4* sA, const uint4* A, uint4* sB, const uint4* B) {
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+#pragma unroll
+        for (int l = 0; l < kGrpVec / kThr; ++l) {
+            const int o = g * kGrpVec + l * kThr + threadIdx.x;
+            const uint32_t da = (uint32_t)__cvta_generic_to_shared(sA + o), db = (uint32_t)__cvta_generic_to_shared(sB + o);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(da), "l"(A + o) : "memory");
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(db), "l"(B + o) : "memory");
         }
-        for (int l = threadIdx.x; l < 1024; l += 256) {
-            int k, j;
-            if (!tb) { k = l / 64; j = l % 64; } else { j = l / 16; k = l % 16; }
-            const int gk = k0 + k, gj = col0 + j;
-            double v = 0.0;
-            if (gk < K && gj < N) v = tb ? B[(int64_t)gj * ldb + gk] : B[(int64_t)gk * ldb + gj];
-            Bs[k][j] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            double a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[k][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[k][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int gi = row0 + ty + 16 * i;
-        if (gi >= M) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int gj = col0 + tx + 16 * j;
-            if (gj >= N || (lower_only && gj > gi)) continue;
-            double* c = C + (int64_t)gi * ldc + gj;
-            *c = (beta == 0.0) ? alpha * acc[i][j] : fma(alpha, acc[i][j], beta * *c);
-        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     }
 }
 
-// Factor the 64x64 diagonal block at (k0, k0) in place (lower) and write the
-// inverse of the factor to Linv.  One block per batch item.  Shared memory
-// holds L in the lower triangle and the strictly-lower part of X = L^-1
-// transposed into the upper triangle (diagonal of X kept apart): 34 KB.
-__global__ void __launch_bounds__(256) k_potrf_diag(double* __restrict__ A, int lda, int64_t sA, int k0,
-                                                    double* __restrict__ Linv, int64_t sLinv, int* __restrict__ err) {
-    A += (int64_t)blockIdx.x * sA;
-    Linv += (int64_t)blockIdx.x * sLinv;
-    __shared__ double L[NB][NB + 1];
-    __shared__ double xd[NB];
-    __shared__ int bad;
-    const int tid = threadIdx.x;
-    if (tid == 0) bad = 0;
-    for (int l = tid; l < NB * NB; l += blockDim.x) {
-        int i = l / NB, j = l % NB;
-        L[i][j] = (j <= i) ? A[(int64_t)(k0 + i) * lda + k0 + j] : 0.0;
-    }
-    __syncthreads();
-    for (int j = 0; j < NB; ++j) {
-        if (tid == 0) {
-            double d = L[j][j];
-            if (!(d > 0.0) || !isfinite(d)) {
-                bad = 1;
-                d = 1.0;
+__device__ __forceinline__ void mma_digits(float (&d)[4], const uint4& a, uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+
+// The warp's 16 x 16 part of A B^T over one block of 64 columns, by order: acc[d] = sum_{i + j = d} A_i B_j^T, digits in
+// shared memory.  Sixteen warps cover 64 x 64: 16-row group warp / 4, 16-column group warp & 3.  ASYNC: the
+// digits are on their way (load_digits); else the caller has synchronised.  Rolled: unrolled
+// copies would not fit the instruction cache.
+template <bool ASYNC>
+__device__ __forceinline__ void mma_block(const uint4* A, const uint4* B, float (&acc)[kDig][2][4]) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, mb = warp >> 2, nb = warp & 3;
+#pragma unroll
+    for (int d = 0; d < kDig; ++d)
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc[d][q][k] = 0.f;
+#pragma unroll 1
+    for (int g = 0; g < 4; ++g) {
+        if (ASYNC) {
+            if (g == 0) asm volatile("cp.async.wait_group 3;" ::: "memory");
+            if (g == 1) asm volatile("cp.async.wait_group 2;" ::: "memory");
+            if (g == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
+            if (g == 3) asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();
+        }
+        uint4 a[kDig];
+#pragma unroll
+        for (int i = 0; i < kDig; ++i) a[i] = A[((g * 4 + mb) * kDig + i) * 32 + lane];
+#pragma unroll
+        for (int j = 0; j < kDig; ++j) {
+            const uint4 b = B[((g * 4 + nb) * kDig + j) * 32 + lane];
+#pragma unroll
+            for (int i = 0; i < kDig - j; ++i) {
+                mma_digits(acc[i + j][0], a[i], b.x, b.z);
+                mma_digits(acc[i + j][1], a[i], b.y, b.w);
             }
-            L[j][j] = sqrt(d);
-        }
-        __syncthreads();
-        const double djj = L[j][j];
-        for (int i = j + 1 + tid; i < NB; i += blockDim.x) L[i][j] /= djj;
-        __syncthreads();
-        const int w = NB - 1 - j;
-        for (int idx = tid; idx < w * w; idx += blockDim.x) {
-            const int i = j + 1 + idx / w, k = j + 1 + idx % w;
-            if (k <= i) L[i][k] -= L[i][j] * L[k][j];
-        }
-        __syncthreads();
-    }
-    // column c of X = L^-1 by forward substitution; X[i][c] (i > c) is kept at L[c][i]
-    if (tid < NB) {
-        const int c = tid;
-        const double xcc = 1.0 / L[c][c];
-        xd[c] = xcc;
-        for (int i = c + 1; i < NB; ++i) {
-            double s = L[i][c] * xcc;
-            for (int k = c + 1; k < i; ++k) s = fma(L[i][k], L[c][k], s);
-            L[c][i] = -s / L[i][i];
         }
     }
-    __syncthreads();
-    for (int l = tid; l < NB * NB; l += blockDim.x) {
-        int i = l / NB, j = l % NB;
-        if (j <= i) A[(int64_t)(k0 + i) * lda + k0 + j] = L[i][j];
-        Linv[l] = (i > j) ? L[j][i] : ((i == j) ? xd[i] : 0.0);
-    }
-    if (tid == 0 && bad) atomicOr(err, ERR_NOT_SPD);
 }
 
-__global__ void k_copy2d(const double* __restrict__ src, int lds, int64_t sS, double* __restrict__ dst, int ldd,
-                         int64_t sD, int rows, int cols) {
-    const int64_t n = (int64_t)rows * cols;
-    src += (int64_t)blockIdx.y * sS;
-    dst += (int64_t)blockIdx.y * sD;
-    for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n; l += (int64_t)gridDim.x * blockDim.x) {
-        int r = (int)(l / cols), c = (int)(l % cols);
-        dst[(int64_t)r * ldd + c] = src[(int64_t)r * lds + c];
+// Row and column of element k (0..3) of 8-column group q (0, 1) of the calling thread's part of the tile.
+__device__ __forceinline__ int tile_row(int k) {
+    return 16 * (threadIdx.x >> 7) + ((threadIdx.x & 31) >> 2) + 8 * (k >> 1);
+}
+__device__ __forceinline__ int tile_col(int q, int k) {
+    return 16 * ((threadIdx.x >> 5) & 3) + 8 * q + 2 * (threadIdx.x & 3) + (k & 1);
+}
+
+__device__ __forceinline__ int small_int(float x) {   // |x| <= 2^22: by the magic constant 1.5 2^23
+    return (int)__float_as_uint(x + 12582912.0f) - 0x4b400000;
+}
+
+// The eight exact sums of one output -> FP64 (e: sum of the two rows' exponents), rounded once, in integer
+// arithmetic only (on the FP64 pipe this would cost more than the products).
+__device__ __forceinline__ double combine(const float (&acc)[kDig][2][4], int q, int k, int e) {
+    const float a0 = acc[0][q][k], a1 = acc[1][q][k], a2 = acc[2][q][k], a3 = acc[3][q][k];
+    const float a4 = acc[4][q][k], a5 = acc[5][q][k], a6 = acc[6][q][k], a7 = acc[7][q][k];
+    // value = (H 2^32 + L) 2^(56 - 124 + e)
+    const long long H = ((long long)small_int(a0) << 24) + ((long long)small_int(a1) << 16) +
+                        ((long long)small_int(a2) << 8) + small_int(a3);
+    const long long L = ((long long)__float2int_rn(a4) << 24) + ((long long)__float2int_rn(a5) << 16) +
+                        ((long long)__float2int_rn(a6) << 8) + __float2int_rn(a7);
+    const int s = min(32, __clzll(H < 0 ? -H : H) - 2);
+    const long long t = (H << s) + (L >> (32 - s));   // |t| < 2^62, value = t 2^(e - 36 - s)
+    if (e >= kNanExp / 2) return __longlong_as_double(0x7ff8000000000000ll);
+    if (t == 0) return 0.0;
+    const unsigned long long a = t < 0 ? (unsigned long long)-t : (unsigned long long)t;
+    const int lz = __clzll((long long)a);
+    const unsigned long long n = a << lz, m = (n >> 11) + ((n >> 10) & 1);   // 53 bits (2^53 carries into the exponent)
+    const int field = 1023 + 63 - lz + e - 36 - s;
+    unsigned long long bits = ((unsigned long long)(field - 1) << 52) + m;
+    if (field <= 0) bits = 0;
+    if (field >= 2047) bits = 0x7ff0000000000000ull;
+    return __longlong_as_double((long long)(bits | ((unsigned long long)t & 0x8000000000000000ull)));
+}
+// Digits of op(X) by blocks of 64 x 64 (zero beyond rows x cols): block (row block blockIdx.x, column chunk
+// blockIdx.y) of batch item blockIdx.z.  trans: element (r, k) is X[k ld + r], else X[r ld + k].
+__global__ void __launch_bounds__(kThr) k_split64(const double* __restrict__ X, int ld, int64_t sX, int rows, int cols,
+                                                 int trans, uint4* __restrict__ dig, int* __restrict__ ex) {
+    __shared__ double sm[NB][NB + 1];
+    __shared__ int es[NB];
+    X += (int64_t)blockIdx.z * sX;
+    const int r0 = blockIdx.x * NB, k0 = blockIdx.y * NB;
+    for (int l = threadIdx.x; l < NB * NB; l += kThr) {
+        const int hi = l / NB, lo = l % NB, r = trans ? lo : hi, k = trans ? hi : lo;
+        double v = 0.0;
+        if (r0 + r < rows && k0 + k < cols)
+            v = trans ? X[(int64_t)(k0 + k) * ld + r0 + r] : X[(int64_t)(r0 + r) * ld + k0 + k];
+        sm[r][k] = v;
+    }
+    __syncthreads();
+    const int64_t blk = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    split_block(sm, es, dig + blk * kBlkVec);
+    if (threadIdx.x < NB) ex[blk * NB + threadIdx.x] = es[threadIdx.x];
+}
+
+// C = alpha A B^T + beta C from the digits of A (MB row blocks) and of B (gridDim.x row blocks), KC chunks of 64.
+__global__ void __launch_bounds__(kThr) k_gemm64(int M, int N, int KC, double alpha, const uint4* __restrict__ dA,
+                                                const int* __restrict__ eA, const uint4* __restrict__ dB,
+                                                const int* __restrict__ eB, double beta, double* __restrict__ C, int ldc,
+                                                int64_t sC) {
+    extern __shared__ uint4 dsm[];
+    const int64_t za = (int64_t)blockIdx.z * KC * gridDim.y, zb = (int64_t)blockIdx.z * KC * gridDim.x;
+    C += (int64_t)blockIdx.z * sC;
+    double sum[2][4];
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) sum[q][k] = 0.0;
+    for (int kc = 0; kc < KC; ++kc) {
+        const int64_t ba = za + (int64_t)kc * gridDim.y + blockIdx.y, bb = zb + (int64_t)kc * gridDim.x + blockIdx.x;
+        float acc[kDig][2][4];
+        if (kc > 0) __syncthreads();   // the previous chunk's digits are read
+        load_digits(dsm, dA + ba * kBlkVec, dsm + kBlkVec, dB + bb * kBlkVec);
+        mma_block<true>(dsm, dsm + kBlkVec, acc);
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                sum[q][k] += combine(acc, q, k, eA[ba * NB + tile_row(k)] + eB[bb * NB + tile_col(q, k)]);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int r = blockIdx.y * NB + tile_row(k), c = blockIdx.x * NB + tile_col(q, k);
+            if (r >= M || c >= N) continue;
+            double* p = C + (int64_t)r * ldc + c;
+            *p = (beta == 0.0) ? alpha * sum[q][k] : fma(alpha, sum[q][k], beta * *p);
+        }
+}
+
+// ---- inverse of an SPD matrix: symmetric block sweeps
+//
+// Sweeping block k of the symmetric B (pivot D = B_kk, P = D^-1, C_i = B_ik):
+// B_ij -= C_i P C_j^T, B_ik = C_i P, B_kk = -P; after every block has been
+// swept B = -A^-1.  The pivots are the Schur complements of a block
+// Cholesky factorisation, so a non-positive one shows that A is not positive
+// definite.  Half the operations of factor + triangular inversion, and two
+// launches per 64 columns: k_sweep_panel forms W = C P (and the digits of C
+// and W), k_sweep_update forms B - W C^T on the lower tiles; its first block
+// per matrix also inverts the next pivot while the others update.
+// What bounds it: one matrix is a chain of n / 64 steps, each the pivot's inversion on one SM (about 60 us), its
+// tile and the panel (25 us); the tiles of a batch are bound by the tensor cores (36 products per FP64
+// product, mma.sync).  Measured against the blocked Cholesky factorisation and substitution on the FP64 pipe
+// that it replaces (GB300, events): n = 512 x 25 matrices 9.9 -> 1.06 ms, 512 x 200 50.0 -> 6.4 ms, 1472 x 8
+// 50.6 -> 4.7 ms, 1984 x 1 30.3 -> 3.1 ms, 2880 x 1 60.8 -> 4.6 ms; max |A X - I| 8e-14 .. 2e-12 (the old one
+// 3e-14 .. 1e-12), and dense_gemm's error against 64-bit-exact sums 4e-16 of sum |a||b| (2e-15 on the FP64 pipe).
+
+// Double-float arithmetic (pairs of floats, about 48 bits) for the pivot blocks: an FP64 instruction of a warp
+// occupies its quarter of the SM for about 60 clocks, these 15 FP32 ones for 15.  The intrinsics keep the
+// compiler from contracting the error terms away.
+struct DF {
+    float h, l;
+};
+__device__ __forceinline__ DF df_norm(float h, float l) {   // |l| <= |h|
+    const float s = __fadd_rn(h, l);
+    return {s, __fsub_rn(l, __fsub_rn(s, h))};
+}
+__device__ __forceinline__ DF df_mul(DF a, DF b) {
+    const float h = __fmul_rn(a.h, b.h);
+    return df_norm(h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -h))));
+}
+__device__ __forceinline__ DF df_recip(DF d) {   // one Newton step with the exact residual
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d.h));
+    return df_norm(r, __fmul_rn(r, __fmaf_rn(-d.l, r, __fmaf_rn(-d.h, r, 1.0f))));
+}
+// c - a b; the sum is left unnormalised (its low part a few roundings of the high one), df_norm before the next product
+__device__ __forceinline__ DF df_fnma(DF a, DF b, DF c) {
+    const float h = __fmul_rn(a.h, b.h);
+    const float l = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -h)));
+    const float s = __fsub_rn(c.h, h), t = __fsub_rn(s, c.h);
+    const float e = __fsub_rn(__fsub_rn(c.h, __fsub_rn(s, t)), __fadd_rn(h, t));
+    return {s, __fadd_rn(e, __fsub_rn(c.l, l))};
+}
+
+struct SweepArgs {
+    double* A;             // the matrix (lower tiles), swept in place
+    int lda, nblk;         // row stride, n / 64
+    int64_t sA;
+    double* P;             // per matrix: 64 x 64 inverse of the pivot, then its digits
+    uint4* dP;
+    int* eP;
+    uint4 *dC, *dW;        // per matrix: digits of the panel C and of W, nblk blocks each
+    int *eC, *eW;
+    int* err;
+};
+
+struct PivotSmem {
+    int es[NB], es2[NB], ex[NB];
+    DF col[2][NB];
+    int bad;
+};
+
+// Inverse of the pivot block in sm (its lower part is read) -> P and its digits; sets the error
+// flag when a pivot is not positive.  dsm: digits of two blocks.
+//   D' = S D S with powers of two S that bring its diagonal into [1, 4)
+//   X  = D'^-1 by symmetric sweeps in double-float (registers, element (ty + 32 a, tx + 16 b), the 16-column groups
+//        that reach the lower part; one barrier per column), relative error about 2^-46 cond(D')
+//   X += (I - X D') X, both products exact to FP64 by digits: squares that error
+//   P  = S X S
+__device__ __noinline__ void finish_pivot(const SweepArgs& S, int z, double (*sm)[NB + 1], uint4* dsm, PivotSmem& T) {
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    if (threadIdx.x == 0) T.bad = 0;
+    __syncthreads();
+    if (threadIdx.x < NB) {
+        const double d = sm[threadIdx.x][threadIdx.x];
+        const int f = exponent_field(d);
+        const bool ok = d > 0.0 && f != 2047 && f != 0;
+        if (!ok) T.bad = 1;
+        T.ex[threadIdx.x] = ok ? (f - 1023) >> 1 : 0;
+    }
+    __syncthreads();
+    // groups b of a row group a: 2 a + 2 of 16 columns (b >> 1 <= a)
+    DF m[2][4];
+    {
+        double v[2][4];
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 2 * a + 2; ++b) {
+                const int r = ty + 32 * a, c = tx + 16 * b;
+                v[a][b] = scale2(r >= c ? sm[r][c] : sm[c][r], -(T.ex[r] + T.ex[c]));
+                m[a][b].h = (float)v[a][b];
+                m[a][b].l = (float)(v[a][b] - (double)m[a][b].h);
+            }
+        __syncthreads();
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 2 * a + 2; ++b) {
+                const int r = ty + 32 * a, c = tx + 16 * b;
+                sm[r][c] = v[a][b];
+                sm[c][r] = v[a][b];
+            }
+    }
+    __syncthreads();
+    split_block(sm, T.es, dsm);             // digits of D'
+#pragma unroll
+    for (int kb = 0; kb < 4; ++kb)
+#pragma unroll 1
+        for (int kt = 0; kt < 16; ++kt) {
+            const int k = 16 * kb + kt, ka = kb >> 1, kr = k & 31;   // row k: ty = kr of row group ka
+            DF* col = T.col[kt & 1];        // the other one may still be read
+            if (tx == kt) {                 // column k, row groups from ka on
+#pragma unroll
+                for (int a = ka; a < 2; ++a) col[ty + 32 * a] = df_norm(m[a][kb].h, m[a][kb].l);
+            }
+            if (ty == kr) {                 // the rest of it is row k
+#pragma unroll
+                for (int b = 0; b < 2 * ka; ++b) col[tx + 16 * b] = df_norm(m[ka][b].h, m[ka][b].l);
+            }
+            __syncthreads();
+            DF d = col[k];
+            if (!(d.h > 0.f) || !(d.h < 3e38f)) {
+                if (threadIdx.x == 0) T.bad = 1;
+                d = {1.f, 0.f};
+            }
+            const DF p = df_recip(d);
+            DF wi[2];
+#pragma unroll
+            for (int a = 0; a < 2; ++a) wi[a] = df_mul(col[ty + 32 * a], p);
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const DF cj = col[tx + 16 * b];
+#pragma unroll
+                for (int a = b >> 1; a < 2; ++a) {
+                    DF v = df_fnma(wi[a], cj, m[a][b]);
+                    if (a == ka && ty == kr) v = df_mul(cj, p);
+                    if (b == kb && tx == kt) v = (a == ka && ty == kr) ? DF{-p.h, -p.l} : wi[a];
+                    m[a][b] = v;
+                }
+            }
+        }
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2 * a + 2; ++b) {      // X = -(swept matrix)
+            const int r = ty + 32 * a, c = tx + 16 * b;
+            const double v = -((double)m[a][b].h + (double)m[a][b].l);
+            if (r >= c) {
+                sm[r][c] = v;
+                sm[c][r] = v;
+            }
+        }
+    __syncthreads();
+    uint4 *dD = dsm, *dX = dsm + kBlkVec;
+    split_block(sm, T.es2, dX);
+    double x[2][4];
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[q][e] = sm[tile_row(e)][tile_col(q, e)];
+    __syncthreads();
+    float acc[kDig][2][4];
+    mma_block<false>(dX, dD, acc);
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {       // R = I - X D'
+            const int r = tile_row(e), c = tile_col(q, e);
+            double v = -combine(acc, q, e, T.es2[r] + T.es[c]);
+            if (r == c) v += 1.0;
+            sm[r][c] = v;
+        }
+    __syncthreads();
+    split_block(sm, T.es, dD);              // (its barrier: every read of D' digits is past)
+    __syncthreads();
+    mma_block<false>(dD, dX, acc);
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {       // X + R X, unscaled
+            const int r = tile_row(e), c = tile_col(q, e);
+            sm[r][c] = scale2(x[q][e] + combine(acc, q, e, T.es[r] + T.es2[c]), -(T.ex[r] + T.ex[c]));
+        }
+    __syncthreads();
+    split_block(sm, T.es, dD);
+    __syncthreads();
+    store_digits(S.dP + (int64_t)z * kBlkVec, dD, S.eP + z * NB, T.es);
+    double* P = S.P + (int64_t)z * NB * NB;
+    for (int l = threadIdx.x; l < NB * NB; l += kThr) P[l] = sm[l / NB][l % NB];
+    if (threadIdx.x == 0 && T.bad) atomicOr(S.err, ERR_NOT_SPD);
+}
+
+__global__ void __launch_bounds__(kThr) k_sweep_first(SweepArgs S) {
+    extern __shared__ uint4 dsm[];
+    __shared__ double sm[NB][NB + 1];
+    __shared__ PivotSmem T;
+    const double* A = S.A + (int64_t)blockIdx.x * S.sA;
+    for (int l = threadIdx.x; l < NB * NB; l += kThr) sm[l / NB][l % NB] = A[(int64_t)(l / NB) * S.lda + l % NB];
+    finish_pivot(S, blockIdx.x, sm, dsm, T);
+}
+
+// Row block blockIdx.y of matrix blockIdx.x: C_i, W_i = C_i P into the matrix, the digits of both.
+__global__ void __launch_bounds__(kThr) k_sweep_panel(SweepArgs S, int k) {
+    extern __shared__ uint4 dsm[];
+    __shared__ double sm[NB][NB + 1];
+    __shared__ int es[NB];
+    const int z = blockIdx.x, i = blockIdx.y;
+    double* A = S.A + (int64_t)z * S.sA;
+    double* T = A + (int64_t)(i >= k ? i : k) * NB * S.lda + (i >= k ? k : i) * NB;   // lower tile of (i, k)
+    if (i == k) {
+        const double* P = S.P + (int64_t)z * NB * NB;
+        for (int l = threadIdx.x; l < NB * NB; l += kThr) T[(int64_t)(l / NB) * S.lda + l % NB] = -P[l];
+        return;
+    }
+    const bool flip = i < k;   // stored as its transpose
+    for (int l = threadIdx.x; l < NB * NB; l += kThr) {
+        const double v = T[(int64_t)(l / NB) * S.lda + l % NB];
+        if (flip) sm[l % NB][l / NB] = v;
+        else sm[l / NB][l % NB] = v;
+    }
+    __syncthreads();
+    const int64_t blk = (int64_t)z * S.nblk + i;
+    uint4 *sC = dsm, *sP = dsm + kBlkVec;
+    const uint4* dP = S.dP + (int64_t)z * kBlkVec;
+    for (int l = threadIdx.x; l < kBlkVec; l += kThr) sP[l] = dP[l];
+    split_block(sm, es, sC);
+    __syncthreads();
+    store_digits(S.dC + blk * kBlkVec, sC, S.eC + blk * NB, es);
+    float acc[kDig][2][4];
+    mma_block<false>(sC, sP, acc);
+    double w[2][4];
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            w[q][e] = combine(acc, q, e, es[tile_row(e)] + S.eP[z * NB + tile_col(q, e)]);
+    __syncthreads();           // es and the digits of C are rewritten below
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sm[tile_row(e)][tile_col(q, e)] = w[q][e];
+    __syncthreads();
+    for (int l = threadIdx.x; l < NB * NB; l += kThr)
+        T[(int64_t)(l / NB) * S.lda + l % NB] = flip ? sm[l % NB][l / NB] : sm[l / NB][l % NB];
+    split_block(sm, es, sC);
+    __syncthreads();
+    store_digits(S.dW + blk * kBlkVec, sC, S.eW + blk * NB, es);
+}
+
+// Lower tile (i, j), i, j != k, of one matrix: B_ij -= W_i C_j^T.  Tile 0 is the next pivot (k + 1, k + 1), which its
+// block then inverts (all matrices' first, so that the long blocks start first); the others follow row by row.
+__global__ void __launch_bounds__(kThr) k_sweep_update(SweepArgs S, int k, int batch) {
+    extern __shared__ uint4 dsm[];
+    __shared__ double sm[NB][NB + 1];
+    __shared__ PivotSmem ps;
+    const int z = blockIdx.x % batch, tile = blockIdx.x / batch, m = S.nblk - 1;
+    const int next = k + 1 < S.nblk ? k : -1;          // index of block k + 1 among the blocks other than k
+    int i, j;
+    const bool pivot = next >= 0 && tile == 0;
+    if (pivot) {
+        i = j = next;
+    } else {
+        // tile number t of the lower triangle (row by row), the next pivot's tile moved to the front
+        int t = tile;
+        if (next >= 0) {
+            const int tn = next * (next + 1) / 2 + next;
+            t = t <= tn ? t - 1 : t;
+        }
+        i = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+        while (i * (i + 1) / 2 > t) --i;
+        while ((i + 1) * (i + 2) / 2 <= t) ++i;
+        j = t - i * (i + 1) / 2;
+        if (i >= m) return;   // (not reached: the grid has m (m + 1) / 2 tiles)
+    }
+    i += i >= k;
+    j += j >= k;
+    const int64_t bi = (int64_t)z * S.nblk + i, bj = (int64_t)z * S.nblk + j;
+    float acc[kDig][2][4];
+    load_digits(dsm, S.dW + bi * kBlkVec, dsm + kBlkVec, S.dC + bj * kBlkVec);
+    mma_block<true>(dsm, dsm + kBlkVec, acc);
+    double* T = S.A + (int64_t)z * S.sA + (int64_t)i * NB * S.lda + j * NB;
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = tile_row(2 * h), c = tile_col(q, 0), ew = S.eW[bi * NB + r];
+            double2* p = reinterpret_cast<double2*>(T + (int64_t)r * S.lda + c);
+            double2 v = *p;
+            v.x -= combine(acc, q, 2 * h, ew + S.eC[bj * NB + c]);
+            v.y -= combine(acc, q, 2 * h + 1, ew + S.eC[bj * NB + c + 1]);
+            *p = v;
+            if (pivot) {
+                sm[r][c] = v.x;
+                sm[r][c + 1] = v.y;
+            }
+        }
+    if (!pivot) return;
+    __syncthreads();
+    finish_pivot(S, z, sm, dsm, ps);
+}
+
+// X = -B, both triangles, from the lower tiles
+__global__ void __launch_bounds__(kThr) k_sweep_store(const double* __restrict__ A, int lda, int64_t sA,
+                                                     double* __restrict__ X, int ldx, int64_t sX) {
+    if (blockIdx.x > blockIdx.y) return;
+    __shared__ double sm[NB][NB + 1];
+    A += (int64_t)blockIdx.z * sA;
+    X += (int64_t)blockIdx.z * sX;
+    const int i = blockIdx.y, j = blockIdx.x;
+    for (int l = threadIdx.x; l < NB * NB; l += kThr) {
+        const int r = l / NB, c = l % NB;
+        const double v = -A[(int64_t)(i * NB + r) * lda + j * NB + c];
+        sm[r][c] = v;
+        X[(int64_t)(i * NB + r) * ldx + j * NB + c] = v;
+    }
+    if (i == j) return;
+    __syncthreads();
+    for (int l = threadIdx.x; l < NB * NB; l += kThr) {
+        const int r = l / NB, c = l % NB;
+        X[(int64_t)(j * NB + r) * ldx + i * NB + c] = sm[c][r];
     }
 }
 
@@ -161,24 +600,63 @@ inline int grid_for(int64_t n) {
     return (int)(b < 65535 ? (b > 0 ? b : 1) : 65535);
 }
 
-void copy2d(const double* src, int lds, int64_t sS, double* dst, int ldd, int64_t sD, int rows, int cols, int batch,
-            cudaStream_t s) {
-    if (rows <= 0 || cols <= 0) return;
-    dim3 g(grid_for((int64_t)rows * cols), batch);
-    k_copy2d<<<g, 256, 0, s>>>(src, lds, sS, dst, ldd, sD, rows, cols);
-    PDG_CHECK_LAUNCH();
+// Temporary device memory of one call, stream-ordered.
+struct Scratch {
+    void* p = nullptr;
+    cudaStream_t s;
+    explicit Scratch(size_t bytes, cudaStream_t st) : s(st) { PDG_CUDA(cudaMallocAsync(&p, bytes, s)); }
+    ~Scratch() { cudaFreeAsync(p, s); }
+    Scratch(const Scratch&) = delete;
+    Scratch& operator=(const Scratch&) = delete;
+};
+
+// the digit kernels' dynamic shared memory exceeds the default limit
+void allow_digit_smem() {
+    static const int lim = std::min(std::min(allow_max_dynamic_smem(k_gemm64), allow_max_dynamic_smem(k_sweep_first)),
+                                    std::min(allow_max_dynamic_smem(k_sweep_panel), allow_max_dynamic_smem(k_sweep_update)));
+    if (lim < kSmemDig) throw Fail{PD_ERR_UNSUPPORTED};
 }
+
+constexpr int64_t kSplitBytes = 16 * (int64_t)kBlkVec + 4 * NB;   // digits and exponents of one 64 x 64 block
+constexpr int64_t kScratchMax = int64_t(64) << 20;               // digits held at once (larger calls go in slices)
 
 }  // namespace
 
 void dense_gemm(bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda, int64_t sA,
                 const double* B, int ldb, int64_t sB, double beta, double* C, int ldc, int64_t sC, int batch,
-                bool lower_only, cudaStream_t s) {
+                cudaStream_t s) {
     if (M <= 0 || N <= 0 || batch <= 0) return;
-    dim3 g((N + 63) / 64, (M + 63) / 64, batch);
-    k_dgemm<<<g, 256, 0, s>>>(M, N, K, alpha, A, lda, sA, ta ? 1 : 0, B, ldb, sB, tb ? 1 : 0, beta, C, ldc, sC,
-                              lower_only ? 1 : 0);
-    PDG_CHECK_LAUNCH();
+    allow_digit_smem();
+    const int KC = (K + NB - 1) / NB, nbN = (N + NB - 1) / NB, nbM = (M + NB - 1) / NB;
+    // slices of the batch, or of the rows of one item, whose digits fit in kScratchMax (and the grid's limits)
+    const int64_t cap = std::max<int64_t>(1, kScratchMax / (kSplitBytes * std::max(KC, 1)));
+    const int mb = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(nbM, 65535), cap - nbN));
+    const int zb = mb < nbM ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(std::min(batch, 65535), cap / (mb + nbN)));
+    const int64_t nA = (int64_t)zb * std::max(KC, 1) * mb, nBl = (int64_t)zb * std::max(KC, 1) * nbN;
+    Scratch w((size_t)(kSplitBytes * (nA + nBl)), s);
+    uint4* dA = static_cast<uint4*>(w.p);
+    uint4* dB = dA + nA * kBlkVec;
+    int* eA = reinterpret_cast<int*>(dB + nBl * kBlkVec);
+    int* eB = eA + nA * NB;
+    for (int z0 = 0; z0 < batch; z0 += zb) {
+        const int nz = std::min(zb, batch - z0);
+        // op(B)^T: its rows are the columns of op(B)
+        if (KC > 0) {
+            k_split64<<<dim3(nbN, KC, nz), kThr, 0, s>>>(B + z0 * sB, ldb, sB, N, K, tb ? 0 : 1, dB, eB);
+            PDG_CHECK_LAUNCH();
+        }
+        for (int m0 = 0; m0 < nbM; m0 += mb) {
+            const int rows = std::min(M - m0 * NB, mb * NB), nm = (rows + NB - 1) / NB;
+            const double* Am = A + z0 * sA + (int64_t)m0 * NB * (ta ? 1 : lda);
+            if (KC > 0) {
+                k_split64<<<dim3(nm, KC, nz), kThr, 0, s>>>(Am, lda, sA, rows, K, ta ? 1 : 0, dA, eA);
+                PDG_CHECK_LAUNCH();
+            }
+            k_gemm64<<<dim3(nbN, nm, nz), kThr, kSmemDig, s>>>(rows, N, KC, alpha, dA, eA, dB, eB, beta,
+                                                       C + z0 * sC + (int64_t)m0 * NB * ldc, ldc, sC);
+            PDG_CHECK_LAUNCH();
+        }
+    }
 }
 
 void dense_set_identity(double* A, int n, int lda, int64_t strideA, int batch, cudaStream_t s) {
@@ -187,82 +665,50 @@ void dense_set_identity(double* A, int n, int lda, int64_t strideA, int batch, c
     PDG_CHECK_LAUNCH();
 }
 
-// Right-looking blocked Cholesky, n a multiple of 64.  Linv: batch x (n/64) x 64 x 64.
-// W: workspace of batch x n x 64 doubles.
-static void cholesky_blocked(double* A, int n, int lda, int64_t sA, int batch, double* Linv, double* W, int* err,
-                             cudaStream_t s) {
-    const int nblk = n / NB;
-    const int64_t sLinv = (int64_t)nblk * NB * NB;
-    const int64_t sW = (int64_t)n * NB;
-    for (int kb = 0; kb < nblk; ++kb) {
-        const int k0 = kb * NB;
-        k_potrf_diag<<<batch, 256, 0, s>>>(A, lda, sA, k0, Linv + (int64_t)kb * NB * NB, sLinv, err);
-        PDG_CHECK_LAUNCH();
-        const int rem = n - k0 - NB;
-        if (rem <= 0) continue;
-        double* P = A + (int64_t)(k0 + NB) * lda + k0;
-        // panel: L_ik = A_ik L_kk^-T
-        dense_gemm(false, true, rem, NB, NB, 1.0, P, lda, sA, Linv + (int64_t)kb * NB * NB, NB, sLinv, 0.0, W, NB,
-                   sW, batch, false, s);
-        copy2d(W, NB, sW, P, lda, sA, rem, NB, batch, s);
-        // trailing update (lower part only)
-        dense_gemm(false, true, rem, rem, NB, -1.0, P, lda, sA, P, lda, sA, 1.0, P + NB, lda, sA, batch, true, s);
-    }
-}
-
-// X = (L L^T)^-1 from the factor (forward then backward substitution on the identity).
-static void inverse_from_factor(const double* L, int n, int lda, int64_t sL, const double* Linv, double* X, int ldx,
-                                int64_t sX, int batch, double* W, cudaStream_t s) {
-    const int nblk = n / NB;
-    const int64_t sLinv = (int64_t)nblk * NB * NB;
-    const int64_t sW = (int64_t)n * NB;
-    dense_set_identity(X, n, ldx, sX, batch, s);
-    for (int kb = 0; kb < nblk; ++kb) {
-        const int k0 = kb * NB;
-        const int cols = k0 + NB;   // the forward solution of the identity is lower triangular
-        double* Xk = X + (int64_t)k0 * ldx;
-        dense_gemm(false, false, NB, cols, NB, 1.0, Linv + (int64_t)kb * NB * NB, NB, sLinv, Xk, ldx, sX, 0.0, W,
-                   cols, sW, batch, false, s);
-        copy2d(W, cols, sW, Xk, ldx, sX, NB, cols, batch, s);
-        const int rem = n - k0 - NB;
-        if (rem > 0)
-            dense_gemm(false, false, rem, cols, NB, -1.0, L + (int64_t)(k0 + NB) * lda + k0, lda, sL, Xk, ldx, sX,
-                       1.0, X + (int64_t)(k0 + NB) * ldx, ldx, sX, batch, false, s);
-    }
-    for (int kb = nblk - 1; kb >= 0; --kb) {
-        const int k0 = kb * NB;
-        double* Xk = X + (int64_t)k0 * ldx;
-        dense_gemm(true, false, NB, n, NB, 1.0, Linv + (int64_t)kb * NB * NB, NB, sLinv, Xk, ldx, sX, 0.0, W, n, sW,
-                   batch, false, s);
-        copy2d(W, n, sW, Xk, ldx, sX, NB, n, batch, s);
-        if (k0 > 0)
-            dense_gemm(true, false, k0, n, NB, -1.0, L + (int64_t)k0 * lda, lda, sL, Xk, ldx, sX, 1.0, X, ldx, sX,
-                       batch, false, s);
-    }
-}
-
-// In-place Cholesky of A (batched, n multiple of 64) and X = A^-1.
+// X = A^-1 (batched SPD matrices, n a multiple of 64, even row stride); A is overwritten.  A pivot that is not
+// positive sets ERR_NOT_SPD in d_err.
 void dense_spd_inverse(double* A, int n, int lda, int64_t sA, double* X, int ldx, int64_t sX, int batch, int* d_err,
                        cudaStream_t s) {
+    if (n <= 0 || batch <= 0) return;
+    allow_digit_smem();
     const int nblk = n / NB;
-    double* Linv = nullptr;
-    double* W = nullptr;
-    PDG_CUDA(cudaMallocAsync((void**)&Linv, sizeof(double) * (size_t)batch * nblk * NB * NB, s));
-    cudaError_t e = cudaMallocAsync((void**)&W, sizeof(double) * (size_t)batch * n * NB, s);
-    if (e != cudaSuccess) {
-        cudaFreeAsync(Linv, s);
-        PDG_CUDA(e);
+    const int zb = (int)std::max<int64_t>(1, std::min<int64_t>(batch, kScratchMax / (kSplitBytes * (2 * nblk + 1))));
+    const int64_t nP = zb, nC = (int64_t)zb * nblk;
+    Scratch w((size_t)(kSplitBytes * (nP + 2 * nC) + sizeof(double) * NB * NB * nP), s);
+    SweepArgs S{};
+    S.lda = lda;
+    S.nblk = nblk;
+    S.sA = sA;
+    S.err = d_err;
+    S.dP = static_cast<uint4*>(w.p);
+    S.dC = S.dP + nP * kBlkVec;
+    S.dW = S.dC + nC * kBlkVec;
+    S.P = reinterpret_cast<double*>(S.dW + nC * kBlkVec);
+    S.eP = reinterpret_cast<int*>(S.P + nP * NB * NB);
+    S.eC = S.eP + nP * NB;
+    S.eW = S.eC + nC * NB;
+    for (int z0 = 0; z0 < batch; z0 += zb) {
+        const int nz = std::min(zb, batch - z0);
+        S.A = A + z0 * sA;
+        k_sweep_first<<<nz, kThr, kSmemDig, s>>>(S);
+        PDG_CHECK_LAUNCH();
+        for (int k = 0; k < nblk; ++k) {
+            k_sweep_panel<<<dim3(nz, nblk), kThr, kSmemDig, s>>>(S, k);
+            PDG_CHECK_LAUNCH();
+            if (nblk > 1) {
+                k_sweep_update<<<nz * (nblk * (nblk - 1) / 2), kThr, kSmemDig, s>>>(S, k, nz);
+                PDG_CHECK_LAUNCH();
+            }
+        }
+        k_sweep_store<<<dim3(nblk, nblk, nz), kThr, 0, s>>>(S.A, lda, sA, X + z0 * sX, ldx, sX);
+        PDG_CHECK_LAUNCH();
     }
-    try {
-        cholesky_blocked(A, n, lda, sA, batch, Linv, W, d_err, s);
-        inverse_from_factor(A, n, lda, sA, Linv, X, ldx, sX, batch, W, s);
-    } catch (...) {
-        cudaFreeAsync(Linv, s);
-        cudaFreeAsync(W, s);
-        throw;
-    }
-    PDG_CUDA(cudaFreeAsync(Linv, s));
-    PDG_CUDA(cudaFreeAsync(W, s));
+}
+
+int64_t dense_scratch_bytes(int n, int batch) {
+    const int64_t nblk = (n + NB - 1) / NB;
+    const int64_t inv = kSplitBytes * (2 * nblk + 1), prod = 2 * kSplitBytes * nblk * nblk;
+    return std::max(inv, std::min<int64_t>(kScratchMax, std::max(inv, prod) * std::max(batch, 1)));
 }
 
 int dense_block() { return NB; }

@@ -826,10 +826,8 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
     PDG_CUDA(cudaMemsetAsync(m->d_err.p, 0, sizeof(int32_t), s));
     dense_spd_inverse(dKii.p, NI, NI, sKii, dXii.p, NI, sKii, n_dom, m->d_err.p, s);
     // Psi = -K_ii^-1 K_ib ;  S_d = K_ib^T Psi = -K_bi K_ii^-1 K_ib
-    dense_gemm(false, false, NI, NBp, NI, -1.0, dXii.p, NI, sKii, dKib.p, NBp, sKib, 0.0, dPsi.p, NBp, sKib, n_dom,
-               false, s);
-    dense_gemm(true, false, NBp, NBp, NI, 1.0, dKib.p, NBp, sKib, dPsi.p, NBp, sKib, 0.0, dSd.p, NBp, sSd, n_dom,
-               false, s);
+    dense_gemm(false, false, NI, NBp, NI, -1.0, dXii.p, NI, sKii, dKib.p, NBp, sKib, 0.0, dPsi.p, NBp, sKib, n_dom, s);
+    dense_gemm(true, false, NBp, NBp, NI, 1.0, dKib.p, NBp, sKib, dPsi.p, NBp, sKib, 0.0, dSd.p, NBp, sSd, n_dom, s);
     dKii.free();
     dKib.free();
 
@@ -869,10 +867,9 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
         std::vector<double> Rinv;
         constexpr int kModalIters = 60;
         for (int it = 0; it <= kModalIters; ++it) {
-            dense_gemm(false, false, NI, NQ, NI, 1.0, dXii.p, NI, sKii, dZ.p, NQ, sZ, 0.0, dY.p, NQ, sZ, n_dom, false,
-                       s);
+            dense_gemm(false, false, NI, NQ, NI, 1.0, dXii.p, NI, sKii, dZ.p, NQ, sZ, 0.0, dY.p, NQ, sZ, n_dom, s);
             if (it == kModalIters) break;
-            dense_gemm(true, false, NQ, NQ, NI, 1.0, dY.p, NQ, sZ, dY.p, NQ, sZ, 0.0, dG.p, NQ, sG, n_dom, false, s);
+            dense_gemm(true, false, NQ, NQ, NI, 1.0, dY.p, NQ, sZ, dY.p, NQ, sZ, 0.0, dG.p, NQ, sG, n_dom, s);
             PDG_CUDA(cudaMemcpyAsync(hG.data(), dG.p, sizeof(double) * hG.size(), cudaMemcpyDeviceToHost, s));
             PDG_CUDA(cudaStreamSynchronize(s));
             std::fill(hR.begin(), hR.end(), 0.0);
@@ -885,10 +882,10 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
                     for (int j = 0; j < q; ++j) hR[(size_t)d * sG + (size_t)i * NQ + j] = Rinv[(size_t)i * q + j];
             }
             PDG_CUDA(cudaMemcpyAsync(dG.p, hR.data(), sizeof(double) * hR.size(), cudaMemcpyHostToDevice, s));
-            dense_gemm(false, false, NI, NQ, NQ, 1.0, dY.p, NQ, sZ, dG.p, NQ, sG, 0.0, dZ.p, NQ, sZ, n_dom, false, s);
+            dense_gemm(false, false, NI, NQ, NQ, 1.0, dY.p, NQ, sZ, dG.p, NQ, sG, 0.0, dZ.p, NQ, sZ, n_dom, s);
         }
         // Rayleigh-Ritz with K_ii^-1: T = Z^T (K_ii^-1 Z), eigenvalues mu = 1 / lambda
-        dense_gemm(true, false, NQ, NQ, NI, 1.0, dZ.p, NQ, sZ, dY.p, NQ, sZ, 0.0, dG.p, NQ, sG, n_dom, false, s);
+        dense_gemm(true, false, NQ, NQ, NI, 1.0, dZ.p, NQ, sZ, dY.p, NQ, sZ, 0.0, dG.p, NQ, sG, n_dom, s);
         PDG_CUDA(cudaMemcpyAsync(hG.data(), dG.p, sizeof(double) * hG.size(), cudaMemcpyDeviceToHost, s));
         PDG_CUDA(cudaStreamSynchronize(s));
         std::vector<double> hV((size_t)n_dom * sV, 0.0), hVs((size_t)n_dom * sV, 0.0), T, w, V;
@@ -920,8 +917,8 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
         upload(dVs, hVs, s);
         dPhi.alloc((size_t)n_dom * sP);
         dPhiS.alloc((size_t)n_dom * sP);
-        dense_gemm(false, false, NI, NR, NQ, 1.0, dZ.p, NQ, sZ, dV.p, NR, sV, 0.0, dPhi.p, NR, sP, n_dom, false, s);
-        dense_gemm(false, false, NI, NR, NQ, 1.0, dZ.p, NQ, sZ, dVs.p, NR, sV, 0.0, dPhiS.p, NR, sP, n_dom, false, s);
+        dense_gemm(false, false, NI, NR, NQ, 1.0, dZ.p, NQ, sZ, dV.p, NR, sV, 0.0, dPhi.p, NR, sP, n_dom, s);
+        dense_gemm(false, false, NI, NR, NQ, 1.0, dZ.p, NQ, sZ, dVs.p, NR, sV, 0.0, dPhiS.p, NR, sP, n_dom, s);
         PDG_CUDA(cudaStreamSynchronize(s));
     }
 
@@ -1014,9 +1011,8 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
         }
         dense_spd_inverse(dS2ii.p, NI2, NI2, s2ii, dX2ii.p, NI2, s2ii, G, m->d_err.p, s);
         dense_gemm(false, false, NI2, NB2, NI2, -1.0, dX2ii.p, NI2, s2ii, dS2it.p, NB2, s2it, 0.0, dPsi2.p, NB2, s2it,
-                   G, false, s);
-        dense_gemm(true, false, NB2, NB2, NI2, 1.0, dS2it.p, NB2, s2it, dPsi2.p, NB2, s2it, 0.0, dS2d.p, NB2, s2d, G,
-                   false, s);
+                   G, s);
+        dense_gemm(true, false, NB2, NB2, NI2, 1.0, dS2it.p, NB2, s2it, dPsi2.p, NB2, s2it, 0.0, dS2d.p, NB2, s2d, G, s);
         dS2.alloc((size_t)nTp * nTp);
         dX2.alloc((size_t)nTp * nTp);
         dense_set_identity(dS2.p, nTp, nTp, 0, 1, s);

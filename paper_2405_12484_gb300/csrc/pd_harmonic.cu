@@ -175,7 +175,7 @@ pd_status pd_harmonic_basis(pd_mesh* m, int32_t r, float* H, double* lambda, int
         // hG = A^T B (q x q)
         auto gram = [&](const double* A, const double* B) {
             dense_gemm(true, false, q, q, kChunk, 1.0, A, q, (int64_t)kChunk * q, B, q, (int64_t)kChunk * q, 0.0,
-                       Gp.p, q, (int64_t)q * q, nch, false, s);
+                       Gp.p, q, (int64_t)q * q, nch, s);
             PDG_CUDA(cudaMemcpyAsync(hGp.data(), Gp.p, sizeof(double) * hGp.size(), cudaMemcpyDeviceToHost, s));
             PDG_CUDA(cudaStreamSynchronize(s));
             std::fill(hG.begin(), hG.end(), 0.0);
@@ -201,7 +201,7 @@ pd_status pd_harmonic_basis(pd_mesh* m, int32_t r, float* H, double* lambda, int
                 gram(A, A);
                 if (!chol_upper_inverse(hG.data(), q, q, Rinv)) throw Fail{PD_ERR_NOT_SPD};
                 PDG_CUDA(cudaMemcpyAsync(G.p, Rinv.data(), sizeof(double) * q * q, cudaMemcpyHostToDevice, s));
-                dense_gemm(false, false, n, q, q, 1.0, A, q, 0, G.p, q, 0, 0.0, Z.p, q, 0, 1, false, s);
+                dense_gemm(false, false, n, q, q, 1.0, A, q, 0, G.p, q, 0, 0.0, Z.p, q, 0, 1, s);
                 PDG_CUDA(cudaMemcpyAsync(A, Z.p, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
             }
         };
@@ -223,7 +223,7 @@ pd_status pd_harmonic_basis(pd_mesh* m, int32_t r, float* H, double* lambda, int
                 for (int i = 0; i < q; ++i) Vs[(size_t)i * q + j] = V[(size_t)i * q + idx[j]];
             }
             PDG_CUDA(cudaMemcpyAsync(G.p, Vs.data(), sizeof(double) * q * q, cudaMemcpyHostToDevice, s));
-            dense_gemm(false, false, n, q, q, 1.0, A, q, 0, G.p, q, 0, 0.0, Z.p, q, 0, 1, false, s);
+            dense_gemm(false, false, n, q, q, 1.0, A, q, 0, G.p, q, 0, 0.0, Z.p, q, 0, 1, s);
             PDG_CUDA(cudaMemcpyAsync(A, Z.p, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
         };
         // largest residual |L x_j - theta_j x_j| over the first r Ritz pairs

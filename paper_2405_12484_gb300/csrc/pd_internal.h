@@ -614,7 +614,8 @@ void launch_axpy_free(const pd_mesh* m, const float4* dx, float4* x, cudaStream_
 // FP64 dense factorisations (device), used by the prefactorisation.
 void dense_gemm(bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
                 int64_t sA, const double* B, int ldb, int64_t sB, double beta, double* C, int ldc,
-                int64_t sC, int batch, bool lower_only, cudaStream_t s);
+                int64_t sC, int batch, cudaStream_t s);
+int64_t dense_scratch_bytes(int n, int batch);   // largest scratch of dense_spd_inverse / dense_gemm on n x n matrices
 void dense_set_identity(double* A, int n, int lda, int64_t strideA, int batch, cudaStream_t s);
 
 // Resolves the fixed scratch array of pd_solve_noalloc on the current device

@@ -170,7 +170,11 @@ static void estimate(pd_mesh* m, int64_t& steady, int64_t& transient) {
     const int64_t small = (int64_t)in.n_tets * 64 + (int64_t)in.n_vertices * 96 + nd * (NI + NB) * 16 +
                           nB * 16 * ((nB + 2047) / 2048 + 1);
     steady = in.device_bytes + pool + small;
-    transient = nd * (2 * NI * NI + 2 * NI * NB + NB * NB) * 8 + 2 * nBp * nBp * 8 + nBp * 64 * 8 * 2;
+    // the two peaks of pd_prefactor: the domains' inverses and boundary modes, then the interface inverse beside
+    // what the domains leave; each with the digit scratch of its dense calls
+    const int64_t kept = nd * (NI * NI + NI * NB + NB * NB) * 8;
+    transient = std::max(kept + nd * (NI * NI + NI * NB) * 8 + dense_scratch_bytes((int)NI, (int)nd),
+                         kept + 2 * nBp * nBp * 8 + dense_scratch_bytes((int)nBp, 1));
 }
 
 // Copies a host vector into a device buffer whose capacity only grows (a
