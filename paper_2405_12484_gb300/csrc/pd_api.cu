@@ -36,8 +36,10 @@ void launch_cast_rowfrag16(const double* src, int lds, int rows, int cols, int t
 bool build_stream_plan(StreamPlan& P, const std::vector<ColDesc>& blocks, int prec, const void* src,
                        cudaStream_t s);
 void reset_stream_plan(StreamPlan& P, cudaStream_t s);
-void launch_prefactor_helpers_scatter_coo(double* S, int ld, const int* r, const int* c, const double* v, int n,
-                                          cudaStream_t s);
+void launch_assemble_K(pd_mesh* m, double inv_h2, cudaStream_t s);
+void launch_domain_blocks(const pd_mesh* m, const int4* dom, const int* bnd, double* Kii, int NI, double* Kib, int NBp,
+                          cudaStream_t s);
+void launch_interface_rows(const pd_mesh* m, double* S, int ld, cudaStream_t s);
 void launch_prefactor_add_block(double* S, int ldS, const double* Sd, int ldSd, const int* bidx, int nb,
                                 cudaStream_t s);
 void launch_cast_block(const double* src, int lds, int rows, int cols, int transpose, int prec, float* dst32,
@@ -636,6 +638,19 @@ pd_status pd_create_mesh(const double* rest_xyz, int32_t n_v, const int32_t* tet
     upload(m->d_inc, inc, s);
     build_local_plan(m, inc_ptr, inc, s);
     upload(m->d_old_of_new, m->old_of_new, s);
+    upload(m->d_K_ptr, m->K_rowptr, s);
+    upload(m->d_K_col, m->K_col, s);
+    m->d_K_val.alloc(m->K_col.size());
+    upload(m->d_kfp_ptr, m->Kfp_rowptr, s);
+    upload(m->d_kfp_col, m->Kfp_col, s);
+    m->d_kfp_val.alloc(m->Kfp_col.size());
+    m->d_mh2.alloc(std::max(m->n_free, 1));
+    std::vector<double> hrest(3 * (size_t)n_v), hmass(m->mass.begin(), m->mass.begin() + m->n_free);
+    for (int32_t i = 0; i < n_v; ++i)
+        for (int c = 0; c < 3; ++c) hrest[3 * (size_t)i + c] = rest_xyz[3 * (size_t)m->old_of_new[i] + c];
+    upload(m->d_rest64, hrest, s);
+    upload(m->d_mass64, hmass, s);
+    m->d_gamma.alloc(2 * (size_t)n_t);
     std::vector<float4> hx(n_v);
     for (int32_t i = 0; i < n_v; ++i) {
         int32_t o = m->old_of_new[i];
@@ -691,11 +706,12 @@ pd_status pd_set_materials(pd_mesh* m, const float* gamma_s, const float* gamma_
         m->gamma_v[t] = gv[m->tet_old_of_new[t]];
         vol[t] = (float)m->vol[t];
     }
-    DBuf<float> dvol, dgs, dgv;
+    DBuf<float> dvol;
     upload(dvol, vol, m->stream);
-    upload(dgs, m->gamma_s, m->stream);
-    upload(dgv, m->gamma_v, m->stream);
-    launch_weights_raw(n_t, dvol.p, dgs.p, dgv.p, m->d_geo.p, m->stream);
+    PDG_CUDA(cudaMemcpyAsync(m->d_gamma.p, m->gamma_s.data(), sizeof(float) * n_t, cudaMemcpyHostToDevice, m->stream));
+    PDG_CUDA(cudaMemcpyAsync(m->d_gamma.p + n_t, m->gamma_v.data(), sizeof(float) * n_t, cudaMemcpyHostToDevice,
+                             m->stream));
+    launch_weights_raw(n_t, dvol.p, m->d_gamma.p, m->d_gamma.p + n_t, m->d_geo.p, m->stream);
     PDG_CUDA(cudaStreamSynchronize(m->stream));
     m->materials_set = true;
     m->prefactored = false;
@@ -735,53 +751,8 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
     const int32_t n_free = m->n_free, n_int = m->n_int, n_B = m->n_B, n_dom = m->n_dom;
     const double inv_h2 = 1.0 / (dt * dt);
 
-    // ---- scalar K over free vertices and the free-pinned block (FP64, host, fixed order)
-    m->K_val.assign(m->K_col.size(), 0.0);
-    m->Kfp_val.assign(m->Kfp_col.size(), 0.0);
-    auto addK = [&](int32_t a, int32_t b, double v) {
-        if (b < n_free) {
-            auto beg = m->K_col.begin() + m->K_rowptr[a], end = m->K_col.begin() + m->K_rowptr[a + 1];
-            m->K_val[std::lower_bound(beg, end, b) - m->K_col.begin()] += v;
-        } else {
-            int32_t p = b - n_free;
-            auto beg = m->Kfp_col.begin() + m->Kfp_rowptr[a], end = m->Kfp_col.begin() + m->Kfp_rowptr[a + 1];
-            m->Kfp_val[std::lower_bound(beg, end, p) - m->Kfp_col.begin()] += v;
-        }
-    };
-    for (int32_t t = 0; t < m->n_t; ++t) {
-        const double* D = &m->Dminv[9 * (size_t)t];
-        double g[4][3];
-        for (int c = 0; c < 3; ++c) {
-            g[1][c] = D[c];
-            g[2][c] = D[3 + c];
-            g[3][c] = D[6 + c];
-            g[0][c] = -(D[c] + D[3 + c] + D[6 + c]);
-        }
-        const double w = m->vol[t] * ((double)m->gamma_s[t] + (double)m->gamma_v[t]);
-        const int32_t* q = &m->tets_new[4 * (size_t)t];
-        for (int a = 0; a < 4; ++a) {
-            if (q[a] >= n_free) continue;
-            for (int b = 0; b < 4; ++b)
-                addK(q[a], q[b], w * (g[a][0] * g[b][0] + g[a][1] * g[b][1] + g[a][2] * g[b][2]));
-        }
-    }
-    for (int32_t i = 0; i < n_free; ++i) addK(i, i, m->mass[i] * inv_h2);
-
-    // per-iteration small arrays
-    {
-        std::vector<float> mh2(std::max(n_free, 1));
-        for (int32_t i = 0; i < n_free; ++i) mh2[i] = (float)(m->mass[i] * inv_h2);
-        upload(m->d_mh2, mh2, s);
-        upload(m->d_kfp_ptr, m->Kfp_rowptr, s);
-        std::vector<int32_t> kc(m->Kfp_col);
-        std::vector<float> kv(m->Kfp_val.size());
-        for (size_t k = 0; k < kv.size(); ++k) kv[k] = (float)m->Kfp_val[k];
-        upload(m->d_kfp_col, kc, s);
-        upload(m->d_kfp_val, kv, s);
-        upload(m->d_K_ptr, m->K_rowptr, s);
-        upload(m->d_K_col, m->K_col, s);
-        upload(m->d_K_val, m->K_val, s);
-    }
+    // ---- scalar K over free vertices, the free-pinned block and m / dt^2 (FP64, device, fixed order)
+    launch_assemble_K(m, inv_h2, s);
 
     // ---- per-domain dense blocks K_ii (padded with identity) and K_ib
     const int nb64 = dense_block();
@@ -793,33 +764,24 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
     const int NI = (int)round_up(max_ni, nb64);
     const int NBp = (int)round_up(max_nb, 8);
     const int64_t sKii = (int64_t)NI * NI, sKib = (int64_t)NI * NBp, sSd = (int64_t)NBp * NBp;
-    std::vector<double> hKii((size_t)n_dom * sKii, 0.0), hKib((size_t)n_dom * sKib, 0.0);
-    {
-        std::vector<int32_t> pos(std::max(n_B, 1), -1);
-        for (int32_t d = 0; d < n_dom; ++d) {
-            double* Kii = &hKii[(size_t)d * sKii];
-            double* Kib = &hKib[(size_t)d * sKib];
-            const auto& bl = m->dom_bnd[d];
-            for (int32_t k = 0; k < (int32_t)bl.size(); ++k) pos[bl[k]] = k;
-            const int32_t off = m->dom_int_off[d], ni = m->dom_n_int[d];
-            for (int32_t r = ni; r < NI; ++r) Kii[(size_t)r * NI + r] = 1.0;
-            for (int32_t r = 0; r < ni; ++r) {
-                const int32_t i = off + r;
-                for (int32_t k = m->K_rowptr[i]; k < m->K_rowptr[i + 1]; ++k) {
-                    const int32_t c = m->K_col[k];
-                    if (c >= off && c < off + ni) Kii[(size_t)r * NI + (c - off)] = m->K_val[k];
-                    else if (c >= n_int) Kib[(size_t)r * NBp + pos[c - n_int]] = m->K_val[k];
-                    else return fail(PD_ERR_BAD_MESH, "internal vertex coupled to another domain's internal vertex");
-                }
-            }
-            for (int32_t k = 0; k < (int32_t)bl.size(); ++k) pos[bl[k]] = -1;
-        }
-    }
+    // boundary index lists of the domains, one after the other
+    std::vector<int32_t> sbidx_off(n_dom + 1, 0), sbidx;
+    for (int32_t d = 0; d < n_dom; ++d) sbidx_off[d + 1] = sbidx_off[d] + (int32_t)m->dom_bnd[d].size();
+    sbidx.reserve(sbidx_off.back());
+    for (int32_t d = 0; d < n_dom; ++d) sbidx.insert(sbidx.end(), m->dom_bnd[d].begin(), m->dom_bnd[d].end());
+    std::vector<int4> hdom(n_dom);
+    for (int32_t d = 0; d < n_dom; ++d)
+        hdom[d] = make_int4(m->dom_int_off[d], m->dom_n_int[d], sbidx_off[d], sbidx_off[d + 1] - sbidx_off[d]);
+    DBuf<int32_t> d_sbidx;
+    DBuf<int4> d_dom;
+    upload(d_sbidx, sbidx, s);
+    upload(d_dom, hdom, s);
     DBuf<double> dKii, dXii, dKib, dPsi, dSd;
-    upload(dKii, hKii, s);
-    upload(dKib, hKib, s);
-    hKii.clear(); hKii.shrink_to_fit();
-    hKib.clear(); hKib.shrink_to_fit();
+    dKii.alloc((size_t)n_dom * sKii);
+    dKib.alloc((size_t)n_dom * sKib);
+    PDG_CUDA(cudaMemsetAsync(dKii.p, 0, sizeof(double) * n_dom * sKii, s));
+    PDG_CUDA(cudaMemsetAsync(dKib.p, 0, sizeof(double) * n_dom * sKib, s));
+    launch_domain_blocks(m, d_dom.p, d_sbidx.p, dKii.p, NI, dKib.p, NBp, s);
     dXii.alloc((size_t)n_dom * sKii);
     dPsi.alloc((size_t)n_dom * sKib);
     dSd.alloc((size_t)n_dom * sSd);
@@ -922,37 +884,15 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
         PDG_CUDA(cudaStreamSynchronize(s));
     }
 
-    // ---- boundary index lists and the reduced interface matrix S = K_BB + sum_d S_d
-    std::vector<int32_t> sbidx_off(n_dom + 1, 0), sbidx;
-    for (int32_t d = 0; d < n_dom; ++d) sbidx_off[d + 1] = sbidx_off[d] + (int32_t)m->dom_bnd[d].size();
-    sbidx.reserve(sbidx_off.back());
-    for (int32_t d = 0; d < n_dom; ++d) sbidx.insert(sbidx.end(), m->dom_bnd[d].begin(), m->dom_bnd[d].end());
-    DBuf<int32_t> d_sbidx;
-    upload(d_sbidx, sbidx, s);
+    // ---- the reduced interface matrix S = K_BB + sum_d S_d
     const int nBp = (int)round_up(std::max(n_B, 1), nb64);
     DBuf<double> dS, dXS;
     const bool two = m->n_groups > 0 && n_B > 0 && !(o.flags & PD_SOLVE_SINGLE_LEVEL);
     if (n_B > 0) {
         dS.alloc((size_t)nBp * nBp);
         dense_set_identity(dS.p, nBp, nBp, 0, 1, s);
-        std::vector<int32_t> cr, cc;
-        std::vector<double> cv;
-        for (int32_t j = 0; j < n_B; ++j) {
-            const int32_t i = n_int + j;
-            for (int32_t k = m->K_rowptr[i]; k < m->K_rowptr[i + 1]; ++k)
-                if (m->K_col[k] >= n_int) {
-                    cr.push_back(j);
-                    cc.push_back(m->K_col[k] - n_int);
-                    cv.push_back(m->K_val[k]);
-                }
-        }
         // diagonal entries of the padding stay 1; real diagonal entries are overwritten
-        DBuf<int32_t> dcr, dcc;
-        DBuf<double> dcv;
-        upload(dcr, cr, s);
-        upload(dcc, cc, s);
-        upload(dcv, cv, s);
-        launch_prefactor_helpers_scatter_coo(dS.p, nBp, dcr.p, dcc.p, dcv.p, (int)cv.size(), s);
+        launch_interface_rows(m, dS.p, nBp, s);
         for (int32_t d = 0; d < n_dom; ++d) {
             const int nbd = (int)m->dom_bnd[d].size();
             if (nbd == 0 || m->dom_n_int[d] == 0) continue;
@@ -1305,6 +1245,10 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
         // the Jacobi diagonal and the Chebyshev weights (Wang 2015) for the
         // spectral radius rho of I - D^-1 K (given, or from 300 power
         // iterations on the similar symmetric I - D^-1/2 K D^-1/2, raised by 1 %)
+        m->K_val.resize(m->K_col.size());
+        PDG_CUDA(cudaMemcpyAsync(m->K_val.data(), m->d_K_val.p, sizeof(double) * m->K_val.size(), cudaMemcpyDeviceToHost,
+                                 s));
+        PDG_CUDA(cudaStreamSynchronize(s));
         std::vector<double> dinv(std::max(n_free, 1), 1.0), sq(std::max(n_free, 1), 1.0);
         for (int32_t i = 0; i < n_free; ++i)
             for (int32_t k = m->K_rowptr[i]; k < m->K_rowptr[i + 1]; ++k)
@@ -1877,6 +1821,7 @@ pd_status pd_get_info(pd_mesh* m, pd_mesh_info* out) {
     bytes += m->d_ax_desc_int.bytes() + m->d_ax_blk_int.bytes() + m->rows_int2.descs.bytes() + m->rows_int2.blk_u.bytes();
     bytes += m->d_ax_blk_back.bytes() + m->d_tc.bytes() + m->d_bidx.bytes();
     bytes += m->d_gat_ptr.bytes() + m->d_gat.bytes() + m->d_cB.bytes() + m->d_part.bytes();
+    bytes += m->d_rest64.bytes() + m->d_mass64.bytes() + m->d_gamma.bytes();
     bytes += m->d_K_ptr.bytes() + m->d_K_col.bytes() + m->d_K_val.bytes() + m->d_r.bytes() + m->d_dx.bytes();
     bytes += m->rows_cond2.descs.bytes() + m->rows_cond2.blk_u.bytes() + m->rows_back2.descs.bytes();
     bytes += m->rows_coarse.descs.bytes() + m->rows_coarse.blk_u.bytes();

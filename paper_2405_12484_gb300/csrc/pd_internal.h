@@ -419,7 +419,7 @@ struct pd_mesh {
     // CSR of the scalar matrix over free vertices (new numbering) and of the free-pinned block
     std::vector<int32_t> K_rowptr, K_col;         // n_free rows, columns < n_free
     std::vector<int32_t> Kfp_rowptr, Kfp_col;     // n_free rows, columns = pinned slot (0..n_pin)
-    std::vector<double> K_val, Kfp_val;
+    std::vector<double> K_val;                    // host copy (modal solve only)
     std::vector<float> gamma_s, gamma_v;          // sorted tet order
 
     // device: geometry and state
@@ -506,6 +506,9 @@ struct pd_mesh {
     // FP64 residual for refinement
     pdg::DBuf<int32_t> d_K_ptr, d_K_col;
     pdg::DBuf<double> d_K_val;
+    // for the assembly of K: rest positions (3 per vertex), masses of the free vertices, gamma_s then gamma_v
+    pdg::DBuf<double> d_rest64, d_mass64;
+    pdg::DBuf<float> d_gamma;
     pdg::DBuf<float4> d_r, d_dx;             // refinement residual / correction (n_free)
 
     // generations of the FP32 state (pd_set_state, pd_step) and of the

@@ -169,7 +169,11 @@ static void estimate(pd_mesh* m, int64_t& steady, int64_t& transient) {
     const int64_t pool = nd * ((NI + NB) * NI + NI * NB) * 4 + nB * ((nB + 7) / 8 * 8) * 4;
     const int64_t small = (int64_t)in.n_tets * 64 + (int64_t)in.n_vertices * 96 + nd * (NI + NB) * 16 +
                           nB * 16 * ((nB + 2047) / 2048 + 1);
-    steady = in.device_bytes + pool + small;
+    // (of `small`, the arrays of K are already there before the prefactorisation)
+    const int64_t early = m->d_K_ptr.bytes() + m->d_K_col.bytes() + m->d_K_val.bytes() + m->d_kfp_ptr.bytes() +
+                          m->d_kfp_col.bytes() + m->d_kfp_val.bytes() + m->d_mh2.bytes() + m->d_rest64.bytes() +
+                          m->d_mass64.bytes() + m->d_gamma.bytes();
+    steady = in.device_bytes - early + pool + std::max(small, early);
     // the two peaks of pd_prefactor: the domains' inverses and boundary modes, then the interface inverse beside
     // what the domains leave; each with the digit scratch of its dense calls
     const int64_t kept = nd * (NI * NI + NI * NB + NB * NB) * 8;
