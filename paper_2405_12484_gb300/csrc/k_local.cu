@@ -3,30 +3,19 @@
 // right-hand-side contributions (in shared memory), and their deterministic
 // sum per vertex into b (or into the residual b - K x).
 //
-// Paper: Sec. 7.1 (local step; R by polar decomposition through the SVD
-// F = U Sigma W^T; V through the three-unknown problem of Eq. vol_pre with
-// targets clamped to >= 0.01), Eq. pd_local, Eq. energy (per-element
-// gamma_s, gamma_v).
+// Paper: Sec. 7.1 (local step; R by polar decomposition, V through the
+// three-unknown problem of Eq. vol_pre with targets clamped to >= 0.01),
+// Eq. pd_local, Eq. energy (per-element gamma_s, gamma_v).  Ordinarily
+// strained elements get both targets as one isotropic function of F^T F;
+// inverted and strongly strained ones by the SVD and the enumeration of the
+// volume problem's candidates (proj3.cuh).
 //
-// SVD: cyclic Jacobi eigen-decomposition of F^T F (Golub & Van Loan,
-// "Matrix Computations", the two-sided symmetric Schur rotation), sorted
-// eigenvectors W in SO(3), then a Givens QR of F W (the structure used by
-// McAdams et al. 2011, "Computing the SVD of 3x3 matrices with minimal
-// branching") so that U in SO(3) and the last singular value carries the
-// sign of det F; a final one-sided Jacobi rotation of the trailing 2x2 block
-// keeps the two smallest singular values accurate when sigma_1 / sigma_3 is
-// beyond the FP32 resolution of F^T F.
-//
-// Volume target: minimise sum (d_i - s_i)^2 s.t. prod d = 1, d_i >= 0.01.
-// KKT: (d_i - s_i) d_i = mu for the free targets.  The smallest target
-// t = d_3 parameterises every candidate root: mu = t (t - s_3) and
-// d_{1,2} = (s_i + sqrt(s_i^2 + 4 mu)) / 2.  On t >= s_3/2 the product is
-// increasing (all roots on the + branch: safeguarded Newton); on
-// [0.01, s_3/2) d_3 is the - root of its quadratic (scan and bisection of
-// every sign change, only where a bound of the product allows a root).  The
-// cheapest candidate is kept; the face with d_3 clamped to 0.01 (d_1 d_2 = 100,
-// the same construction) is tried when the first face has no feasible point
-// or a - root under the clamp; failing both, d = (1e4, 0.01, 0.01).
+// What bounds it: with the SVD path for every element the kernel was bound
+// by instruction issue (1,050 thread instructions per element; 25.7 us for
+// 390,000 elements, ncu, cold caches).  Now 18.6 us (640 instructions with
+// the vertex sums): the latency of the loads (long-scoreboard stalls, 39 %
+// of the warps resident, 2.5 waves); 64-tet blocks, 96-tet blocks and 48
+// registers measure within 0.5 % of this.
 //
 // The serving loop runs the same block code over every resident request in
 // one launch (k_b_local_assemble, k_b_assemble_shared).
@@ -42,37 +31,60 @@ namespace {
 
 using namespace proj;
 
-__global__ void __launch_bounds__(256) k_project(const float* __restrict__ Fin, int n, float* __restrict__ Rout,
-                                                 float* __restrict__ Vout, float* __restrict__ sout) {
-    int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    float F[3][3];
+// Rotation and volume targets of n matrices.  390,000 of them: 25.5 us a call before (one matrix per thread read in
+// place, SVD of each), 20-24 us now, of which the host's part is 19; bound by instruction issue (70 %).
+// Matrices go through shared memory: consecutive threads read and write consecutive floats of the 36-byte records
+// (read in place, a warp's loads touch nine times the lines), and the odd record length is free of bank conflicts.
+constexpr int kProjThreads = 128;
+
+__global__ void __launch_bounds__(kProjThreads) k_project(const float* __restrict__ Fin, int n, float* __restrict__ Rout,
+                                                          float* __restrict__ Vout, float* __restrict__ sout) {
+    __shared__ float buf[9 * kProjThreads];
+    const int64_t e0 = (int64_t)blockIdx.x * kProjThreads;
+    const int ne = (int)min((int64_t)kProjThreads, n - e0), tid = threadIdx.x;
+    for (int l = tid; l < 9 * ne; l += kProjThreads) buf[l] = Fin[9 * e0 + l];
+    __syncthreads();
+    float F[3][3], R[3][3], V[3][3], s[3];
+    const int me = min(tid, ne - 1);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) F[i][j] = Fin[9 * (int64_t)e + 3 * i + j];
-    float U[3][3], W[3][3], s[3], d[3], P[3][3];
-    svd3(F, U, s, W);
-    if (sout) {
-        sout[3 * (int64_t)e] = s[0];
-        sout[3 * (int64_t)e + 1] = s[1];
-        sout[3 * (int64_t)e + 2] = s[2];
+        for (int j = 0; j < 3; ++j) F[i][j] = buf[9 * me + 3 * i + j];
+    Strain S;
+    if (strain_of<true>(F, S)) {
+        strain_apply<false>(F, S, 1.f, 0.f, R);
+        strain_apply<false>(F, S, 0.f, 1.f, V);
+        s[0] = S.s1;
+        s[1] = S.s2;
+        s[2] = S.s3;
+    } else {
+        float U[3][3], W[3][3], d[3];
+        const float one[3] = {1.f, 1.f, 1.f};
+        svd3(F, U, s, W);
+        udwt(U, one, W, R);
+        volume_targets(s, d);
+        udwt(U, d, W, V);
     }
     if (Rout) {
-        const float one[3] = {1.f, 1.f, 1.f};
-        udwt(U, one, W, P);
+        __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) Rout[9 * (int64_t)e + 3 * i + j] = P[i][j];
+        for (int i = 0; i < 9; ++i) buf[9 * tid + i] = R[i / 3][i % 3];
+        __syncthreads();
+        for (int l = tid; l < 9 * ne; l += kProjThreads) Rout[9 * e0 + l] = buf[l];
     }
     if (Vout) {
-        volume_targets(s, d);
-        udwt(U, d, W, P);
+        __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
+        for (int i = 0; i < 9; ++i) buf[9 * tid + i] = V[i / 3][i % 3];
+        __syncthreads();
+        for (int l = tid; l < 9 * ne; l += kProjThreads) Vout[9 * e0 + l] = buf[l];
+    }
+    if (sout) {
+        __syncthreads();
 #pragma unroll
-            for (int j = 0; j < 3; ++j) Vout[9 * (int64_t)e + 3 * i + j] = P[i][j];
+        for (int i = 0; i < 3; ++i) buf[3 * tid + i] = s[i];
+        __syncthreads();
+        for (int l = tid; l < 3 * ne; l += kProjThreads) sout[3 * e0 + l] = buf[l];
     }
 }
 
@@ -83,6 +95,17 @@ __global__ void __launch_bounds__(256) k_project(const float* __restrict__ Fin, 
 struct LocalIn {
     float4 r1, r2, r3, x0, x1, x2, x3;
 };
+
+// The general element (inverted, strongly strained), out of line so that the usual one keeps its registers.
+template <bool RESID>
+__device__ __noinline__ void svd_apply(const float (&F)[3][3], float ws, float wv, float (&P)[3][3]) {
+    float U[3][3], W[3][3], s[3], d[3], c[3];
+    svd3(F, U, s, W);
+    volume_targets(s, d);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) c[i] = RESID ? ws * (1.f - s[i]) + wv * (d[i] - s[i]) : ws + wv * d[i];
+    udwt(U, c, W, P);
+}
 
 // Per-tet corner terms f_c = P g_c with P = U diag(c) W^T: the RHS form
 // c_i = w_s + w_v d_i (P = w_s R + w_v V), or the residual form
@@ -101,14 +124,11 @@ __device__ __forceinline__ void local_corners(const LocalIn& L, float (&out)[4][
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = 0; j < 3; ++j) F[i][j] = e1[i] * g1[j] + e2[i] * g2[j] + e3[i] * g3[j];
-    float U[3][3], W[3][3], s[3], d[3], P[3][3];
-    svd3(F, U, s, W);
-    volume_targets(s, d);
+    float P[3][3];
     const float ws = L.r1.w, wv = L.r2.w;
-    float c[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) c[i] = RESID ? ws * (1.f - s[i]) + wv * (d[i] - s[i]) : ws + wv * d[i];
-    udwt(U, c, W, P);
+    Strain S;
+    if (strain_of<false>(F, S)) strain_apply<RESID>(F, S, ws, wv, P);
+    else svd_apply<RESID>(F, ws, wv, P);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         out[1][i] = P[i][0] * g1[0] + P[i][1] * g1[1] + P[i][2] * g1[2];
@@ -384,7 +404,7 @@ void launch_b_assemble_shared(const BatchSlot* slots, const int* off, int n_slot
 
 void launch_project(const float* F, int n, float* R, float* V, float* sig, cudaStream_t s) {
     if (n <= 0) return;
-    k_project<<<(n + 255) / 256, 256, 0, s>>>(F, n, R, V, sig);
+    k_project<<<(n + kProjThreads - 1) / kProjThreads, kProjThreads, 0, s>>>(F, n, R, V, sig);
     PDG_CHECK_LAUNCH();
 }
 

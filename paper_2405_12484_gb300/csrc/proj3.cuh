@@ -369,6 +369,179 @@ static __device__ __forceinline__ void volume_targets(const float (&s)[3], float
     dd[2] = kClamp;
 }
 
+// ---- targets of ordinarily strained elements without an SVD
+//
+// With C = F^T F, sigma_i = sqrt(lambda_i) and the all-"+" root of the
+// volume problem, d_i (d_i - sigma_i) = mu, so d_i / sigma_i =
+// (1 + sqrt(1 + 4 mu / lambda_i)) / 2 and
+//   w_s R + w_v V = F h(C),   h(l) = w_s l^-1/2 + w_v (1 + sqrt(1 + 4 mu / l)) / 2
+// (residual form: h(l) - w_s - w_v).  h(C) is the quadratic that
+// interpolates h at the three eigenvalues, in Newton's form; its divided
+// differences have closed forms without cancellation (l^-1/2 and
+// sqrt(1 + 4 mu / l) differ by l_a - l_b times a sum of positive terms), so
+// coincident eigenvalues, the rest state, need no special case, and an error
+// of an eigenvalue enters only times the squared spread of the others.  The
+// eigenvalues come from the trigonometric solution of the characteristic
+// polynomial of C - I (Smith, "Eigenvalues of a symmetric 3 x 3 matrix",
+// CACM 4, 1961).
+//
+// Used where det F > 0, J = sigma_1 sigma_2 sigma_3 < 1.9 and lambda_1 <=
+// 6 lambda_3, lambda_3 >= 0.04: for J < 2 the all-"+" root exists and no "-"
+// root does (their product is at most J / 2), every target exceeds sigma_3 / 2,
+// far above the clamp, and the squared condition number that C brings stays
+// within a few roundings of the SVD.  Everything else takes svd3 and
+// volume_targets.  About 300 instructions against 1,050.
+struct Strain {
+    float e00, e01, e02, e11, e12, e22;   // C - I
+    float l1, l2, l3, e1, e2;             // eigenvalues (descending), l - 1 of the first two
+    float s1, s2, s3, i1, i2, i3;         // singular values and their reciprocals
+    float mu, q1, q2, q3, r1, r3;         // root, sqrt(1 + 4 mu / l), sqrt(l + 4 mu)
+};
+
+#define PDG_HD __host__ __device__ __forceinline__
+// The three eigenvalues of the symmetric K (trace 0) given approximately, k (descending): the trigonometric solution
+// is accurate to sqrt(rounding) only where two coincide, which h(C) does not mind but singular values do.  The
+// eigenvector of the isolated end, then the 2 x 2 block on its complement.
+static PDG_HD void polish_eigenvalues(float k0, float k1, float k2, float k01, float k02, float k12, float (&k)[3]) {
+    const bool top = k[0] - k[1] >= k[1] - k[2];
+    const float x = top ? k[0] : k[2];
+    const float r0[3] = {k0 - x, k01, k02}, r1[3] = {k01, k1 - x, k12}, r2[3] = {k02, k12, k2 - x};
+    float v[3] = {r0[1] * r1[2] - r0[2] * r1[1], r0[2] * r1[0] - r0[0] * r1[2], r0[0] * r1[1] - r0[1] * r1[0]};
+    const float b[3] = {r0[1] * r2[2] - r0[2] * r2[1], r0[2] * r2[0] - r0[0] * r2[2], r0[0] * r2[1] - r0[1] * r2[0]};
+    const float c[3] = {r1[1] * r2[2] - r1[2] * r2[1], r1[2] * r2[0] - r1[0] * r2[2], r1[0] * r2[1] - r1[1] * r2[0]};
+    float n = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+    const float nb = b[0] * b[0] + b[1] * b[1] + b[2] * b[2], nc = c[0] * c[0] + c[1] * c[1] + c[2] * c[2];
+    if (nb > n) { n = nb; v[0] = b[0]; v[1] = b[1]; v[2] = b[2]; }
+    if (nc > n) { n = nc; v[0] = c[0]; v[1] = c[1]; v[2] = c[2]; }
+    if (!(n > 1e-36f)) return;   // K is zero to rounding
+    const float in = rsqrtf(n);
+    v[0] *= in;
+    v[1] *= in;
+    v[2] *= in;
+    // orthonormal complement (Duff et al., "Building an orthonormal basis, revisited", JCGT 6, 2017)
+    const float sg = copysignf(1.f, v[2]), a = -1.f / (sg + v[2]), d = v[0] * v[1] * a;
+    const float u[3] = {1.f + sg * v[0] * v[0] * a, sg * d, -sg * v[0]};
+    const float w[3] = {d, sg + v[1] * v[1] * a, -v[1]};
+    const float Ku[3] = {k0 * u[0] + k01 * u[1] + k02 * u[2], k01 * u[0] + k1 * u[1] + k12 * u[2],
+                         k02 * u[0] + k12 * u[1] + k2 * u[2]};
+    const float Kw[3] = {k0 * w[0] + k01 * w[1] + k02 * w[2], k01 * w[0] + k1 * w[1] + k12 * w[2],
+                         k02 * w[0] + k12 * w[1] + k2 * w[2]};
+    const float uu = u[0] * Ku[0] + u[1] * Ku[1] + u[2] * Ku[2], ww = w[0] * Kw[0] + w[1] * Kw[1] + w[2] * Kw[2];
+    const float uw = u[0] * Kw[0] + u[1] * Kw[1] + u[2] * Kw[2];
+    const float hm = 0.5f * (uu + ww), hd = 0.5f * (uu - ww), g = sqrtf(hd * hd + uw * uw);
+    const float iso = -(uu + ww);
+    if (top) { k[0] = iso; k[1] = hm + g; k[2] = hm - g; }
+    else { k[0] = hm + g; k[1] = hm - g; k[2] = iso; }
+}
+
+template <bool POLISH>
+static PDG_HD bool strain_of(const float (&F)[3][3], Strain& S) {
+    S.e00 = F[0][0] * F[0][0] + F[1][0] * F[1][0] + (F[2][0] * F[2][0] - 1.f);
+    S.e11 = F[0][1] * F[0][1] + F[1][1] * F[1][1] + (F[2][1] * F[2][1] - 1.f);
+    S.e22 = F[0][2] * F[0][2] + F[1][2] * F[1][2] + (F[2][2] * F[2][2] - 1.f);
+    S.e01 = F[0][0] * F[0][1] + F[1][0] * F[1][1] + F[2][0] * F[2][1];
+    S.e02 = F[0][0] * F[0][2] + F[1][0] * F[1][2] + F[2][0] * F[2][2];
+    S.e12 = F[0][1] * F[0][2] + F[1][1] * F[1][2] + F[2][1] * F[2][2];
+    const float det = F[0][0] * (F[1][1] * F[2][2] - F[1][2] * F[2][1]) - F[0][1] * (F[1][0] * F[2][2] - F[1][2] * F[2][0]) +
+                      F[0][2] * (F[1][0] * F[2][1] - F[1][1] * F[2][0]);
+    const float m = (S.e00 + S.e11 + S.e22) * (1.f / 3.f);
+    const float k0 = S.e00 - m, k1 = S.e11 - m, k2 = S.e22 - m;
+    const float a = S.e01 * S.e01, b = S.e02 * S.e02, c = S.e12 * S.e12;
+    const float p = fmaxf((k0 * k0 + k1 * k1 + k2 * k2 + 2.f * (a + b + c)) * (1.f / 6.f), 1e-30f);
+    const float ip = rsqrtf(p), sp2 = 2.f * p * ip;
+    const float half = 0.5f * (k0 * (k1 * k2 - c) + 2.f * S.e01 * S.e02 * S.e12 - b * k1 - a * k2);
+    const float phi = acosf(fminf(fmaxf(half * ip * ip * ip, -1.f), 1.f)) * (1.f / 3.f);
+    float sn, cs;
+#ifdef __CUDA_ARCH__
+    __sincosf(phi, &sn, &cs);
+#else
+    sn = sinf(phi);
+    cs = cosf(phi);
+#endif
+    float k[3] = {sp2 * cs, 0.f, -sp2 * (0.5f * cs + 0.8660254f * sn)};
+    k[1] = -(k[0] + k[2]);
+    if (POLISH) polish_eigenvalues(k0, k1, k2, S.e01, S.e02, S.e12, k);
+    const float e3 = m + k[2];
+    S.e1 = m + k[0];
+    S.e2 = m + k[1];
+    S.l1 = 1.f + S.e1;
+    S.l2 = 1.f + S.e2;
+    S.l3 = 1.f + e3;
+    // J^2 - 1 from the strains
+    const float j21 = S.e1 + S.e2 + e3 + (S.e1 * S.e2 + S.e1 * e3 + S.e2 * e3) + S.e1 * S.e2 * e3;
+    if (!(det > 0.f && S.l3 >= 0.04f && S.l1 <= 6.f * S.l3 && j21 < 2.6f)) return false;
+    S.i1 = rsqrtf(S.l1);
+    S.i2 = rsqrtf(S.l2);
+    S.i3 = rsqrtf(S.l3);
+    S.s1 = S.l1 * S.i1;
+    S.s2 = S.l2 * S.i2;
+    S.s3 = S.l3 * S.i3;
+    // product of the targets = 1 by Newton's method in mu, from the root of the element scaled uniformly
+    // (d = f sigma, f = J^-1/3; f - 1 by a Pade approximant in J^2 - 1, exact to first order): off by the
+    // square of the shear only
+    const float lo = -0.24f * S.l3, fm = -j21 / (6.f + j21 * (3.5f - 0.486f * j21));
+    float mu = 3.f * (1.f + fm) * fm / (S.i1 * S.i1 + S.i2 * S.i2 + S.i3 * S.i3);
+    mu = fmaxf(mu, lo);
+    float r1, r2, r3;
+#ifdef __CUDA_ARCH__
+#pragma unroll 1
+#endif
+    for (int it = 0;; ++it) {
+        r1 = sqrtf(S.l1 + 4.f * mu);
+        r2 = sqrtf(S.l2 + 4.f * mu);
+        r3 = sqrtf(S.l3 + 4.f * mu);
+        const float d1 = 0.5f * (S.s1 + r1), d2 = 0.5f * (S.s2 + r2), d3 = 0.5f * (S.s3 + r3);
+        const float pr = d1 * d2 * d3, v = pr - 1.f;
+        if (fabsf(v) <= 3e-7f) break;
+        if (it == 8) return false;
+        const float x1 = r1 * d1, x2 = r2 * d2, x3 = r3 * d3;   // d ln d_i / d mu = 1 / x_i
+        mu = fmaxf(mu - v * (x1 * x2 * x3) / (pr * (x2 * x3 + x1 * x3 + x1 * x2)), lo);
+        if (fabsf(v) <= 1e-5f) {   // the step squares it (times at most some 500, where r3 is small): below rounding
+            r1 = sqrtf(S.l1 + 4.f * mu);
+            r2 = sqrtf(S.l2 + 4.f * mu);
+            r3 = sqrtf(S.l3 + 4.f * mu);
+            break;
+        }
+    }
+    S.mu = mu;
+    S.r1 = r1;
+    S.r3 = r3;
+    S.q1 = r1 * S.i1;
+    S.q2 = r2 * S.i2;
+    S.q3 = r3 * S.i3;
+    return true;
+}
+
+// P = F h(C) for weights (w_s, w_v); RESID: h - w_s - w_v.
+template <bool RESID>
+static PDG_HD void strain_apply(const float (&F)[3][3], const Strain& S, float ws, float wv, float (&P)[3][3]) {
+    const float s12 = S.s1 + S.s2, s23 = S.s2 + S.s3, s13 = S.s1 + S.s3, i12 = S.i1 * S.i2, i123 = i12 * S.i3;
+    const float q12 = S.q1 + S.q2, q23 = S.q2 + S.q3;
+    const float h1 = RESID ? wv * (2.f * S.mu * S.i1 * S.i1) / (1.f + S.q1) - ws * S.e1 * S.i1 / (1.f + S.s1)
+                           : ws * S.i1 + 0.5f * wv * (1.f + S.q1);
+    const float h12 = -(ws * i12 / s12 + wv * (2.f * S.mu * i12 * i12) / q12);
+    const float h123 = ws * i123 * (S.s1 + s23) / (s12 * s23 * s13) +
+                       wv * (2.f * S.mu * i123 * i123) * ((S.l1 + S.l3 + 4.f * S.mu) / (S.s1 * S.r1 + S.s3 * S.r3) + S.q2) /
+                           (q12 * q23);
+    // M = h1 + X (h12 + h123 Y), X = C - l1, Y = C - l2
+    const float x0 = S.e00 - S.e1, x1 = S.e11 - S.e1, x2 = S.e22 - S.e1;
+    const float y0 = h12 + h123 * (S.e00 - S.e2), y1 = h12 + h123 * (S.e11 - S.e2), y2 = h12 + h123 * (S.e22 - S.e2);
+    const float z01 = h123 * S.e01, z02 = h123 * S.e02, z12 = h123 * S.e12;
+    const float m00 = h1 + x0 * y0 + S.e01 * z01 + S.e02 * z02;
+    const float m11 = h1 + x1 * y1 + S.e01 * z01 + S.e12 * z12;
+    const float m22 = h1 + x2 * y2 + S.e02 * z02 + S.e12 * z12;
+    const float m01 = x0 * z01 + S.e01 * y1 + S.e02 * z12;
+    const float m02 = x0 * z02 + S.e01 * z12 + S.e02 * y2;
+    const float m12 = S.e01 * z02 + x1 * z12 + S.e12 * y2;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        P[i][0] = F[i][0] * m00 + F[i][1] * m01 + F[i][2] * m02;
+        P[i][1] = F[i][0] * m01 + F[i][1] * m11 + F[i][2] * m12;
+        P[i][2] = F[i][0] * m02 + F[i][1] * m12 + F[i][2] * m22;
+    }
+}
+#undef PDG_HD
+
 // P = U diag(c) W^T
 static __device__ __forceinline__ void udwt(const float (&U)[3][3], const float (&c)[3], const float (&W)[3][3],
                                      float (&P)[3][3]) {
