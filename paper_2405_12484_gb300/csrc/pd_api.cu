@@ -1821,6 +1821,7 @@ pd_status pd_get_info(pd_mesh* m, pd_mesh_info* out) {
     bytes += m->d_ax_desc_int.bytes() + m->d_ax_blk_int.bytes() + m->rows_int2.descs.bytes() + m->rows_int2.blk_u.bytes();
     bytes += m->d_ax_blk_back.bytes() + m->d_tc.bytes() + m->d_bidx.bytes();
     bytes += m->d_gat_ptr.bytes() + m->d_gat.bytes() + m->d_cB.bytes() + m->d_part.bytes();
+    for (const auto& buf : m->d_io) bytes += buf.bytes();
     bytes += m->d_rest64.bytes() + m->d_mass64.bytes() + m->d_gamma.bytes();
     bytes += m->d_K_ptr.bytes() + m->d_K_col.bytes() + m->d_K_val.bytes() + m->d_r.bytes() + m->d_dx.bytes();
     bytes += m->rows_cond2.descs.bytes() + m->rows_cond2.blk_u.bytes() + m->rows_back2.descs.bytes();
@@ -1852,12 +1853,9 @@ pd_status pd_local_rhs(pd_mesh* m, const float* x, const float* y, float* b) {
     PD_API_BEGIN
     pdg::AllocStreamScope alloc_scope(m->stream);
     cudaStream_t s = m->stream;
-    DBuf<float4> xi, yi, by0, bb, frc;
-    xi.alloc(m->n_v);
-    yi.alloc(m->n_v);
-    by0.alloc(std::max(m->n_free, 1));
-    bb.alloc(m->n_v);
-    frc.alloc(4 * (size_t)m->n_t);
+    for (auto& buf : m->d_io)
+        if (!buf.p) buf.alloc(m->n_v);
+    DBuf<float4>&xi = m->d_io[0], &yi = m->d_io[1], &by0 = m->d_io[2], &bb = m->d_io[3];
     launch_gather_in(m, x, xi.p, s);
     launch_gather_in(m, y, yi.p, s);
     // pinned positions for the K_fp term come from x
@@ -1878,20 +1876,16 @@ pd_status pd_solve(pd_mesh* m, const float* r, float* x) {
     PD_API_BEGIN
     pdg::AllocStreamScope alloc_scope(m->stream);
     cudaStream_t s = m->stream;
-    DBuf<float4> ri, xi;
-    ri.alloc(m->n_v);
-    xi.alloc(m->n_v);
+    for (int k = 0; k < (m->refine > 0 ? 4 : 2); ++k)
+        if (!m->d_io[k].p) m->d_io[k].alloc(m->n_v);
+    DBuf<float4>&ri = m->d_io[0], &xi = m->d_io[1], &rr = m->d_io[2], &dx = m->d_io[3];
     PDG_CUDA(cudaMemsetAsync(xi.p, 0, sizeof(float4) * m->n_v, s));
     launch_gather_in(m, r, ri.p, s);
     launch_dd_solve(m, ri.p, xi.p, s, false);
     for (int k = 0; k < m->refine; ++k) {
-        DBuf<float4> rr, dx;
-        rr.alloc(std::max(m->n_free, 1));
-        dx.alloc(m->n_v);
         launch_residual(m, ri.p, xi.p, rr.p, s);
         launch_dd_solve(m, rr.p, dx.p, s, false);
         launch_axpy_free(m, dx.p, xi.p, s);
-        PDG_CUDA(cudaStreamSynchronize(s));
     }
     launch_scatter_out(m, xi.p, x, 1, s);
     PDG_CUDA(cudaStreamSynchronize(s));
