@@ -7,13 +7,14 @@
 // three-unknown problem of Eq. vol_pre with targets clamped to >= 0.01),
 // Eq. pd_local, Eq. energy (per-element gamma_s, gamma_v).  Ordinarily
 // strained elements get both targets as one isotropic function of F^T F;
-// inverted and strongly strained ones by the SVD and the enumeration of the
-// volume problem's candidates (proj3.cuh).
+// inverted and strongly strained ones, and every one in the frames of the
+// direct form (see local_corners), by the SVD and the enumeration of the volume
+// problem's candidates (proj3.cuh).
 //
 // What bounds it: with the SVD path for every element the kernel was bound
 // by instruction issue (1,050 thread instructions per element; 25.7 us for
-// 390,000 elements, ncu, cold caches).  Now 18.6 us (640 instructions with
-// the vertex sums): the latency of the loads (long-scoreboard stalls, 39 %
+// 390,000 elements, ncu, cold caches).  Without it 18.6 us (640 instructions
+// with the vertex sums): the latency of the loads (long-scoreboard stalls, 39 %
 // of the warps resident, 2.5 waves); 64-tet blocks, 96-tet blocks and 48
 // registers measure within 0.5 % of this.
 //
@@ -96,22 +97,36 @@ struct LocalIn {
     float4 r1, r2, r3, x0, x1, x2, x3;
 };
 
-// The general element (inverted, strongly strained), out of line so that the usual one keeps its registers.
+// P = U diag(c) W^T for any element.
 template <bool RESID>
-__device__ __noinline__ void svd_apply(const float (&F)[3][3], float ws, float wv, float (&P)[3][3]) {
-    float U[3][3], W[3][3], s[3], d[3], c[3];
+__device__ __forceinline__ void svd_targets(const float (&F)[3][3], float ws, float wv, float (&P)[3][3]) {
+    float U[3][3], W[3][3], s[3], d[3];
     svd3(F, U, s, W);
     volume_targets(s, d);
+    float c[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) c[i] = RESID ? ws * (1.f - s[i]) + wv * (d[i] - s[i]) : ws + wv * d[i];
     udwt(U, c, W, P);
+}
+
+// The same out of line, for the rare element beside the fast path (which keeps its registers).
+template <bool RESID>
+__device__ __noinline__ void svd_targets_rare(const float (&F)[3][3], float ws, float wv, float (&P)[3][3]) {
+    svd_targets<RESID>(F, ws, wv, P);
 }
 
 // Per-tet corner terms f_c = P g_c with P = U diag(c) W^T: the RHS form
 // c_i = w_s + w_v d_i (P = w_s R + w_v V), or the residual form
 // c_i = w_s (1 - s_i) + w_v (d_i - s_i) (P = w_s (R - F) + w_v (V - F), the
 // elastic part of b - K x without cancellation: F = U diag(s) W^T).
-template <bool RESID>
+//
+// FAST: the SVD-free targets (strain_of).  The frames of the direct form (x =
+// S(b), FP32) do not use them: there the rounding of every local step enters
+// the positions at full size (an ulp of a 2 m garment is 4e-5 m/s of its
+// velocity), and their trajectories stay what they were.  In the
+// correction form it only enters the shrinking correction.  Frame of the 390K
+// shell with / without: BF16 1.57 / 1.67 ms (FP32 would gain 2.01 -> 1.98).
+template <bool RESID, bool FAST>
 __device__ __forceinline__ void local_corners(const LocalIn& L, float (&out)[4][3]) {
     const float e1[3] = {L.x1.x - L.x0.x, L.x1.y - L.x0.y, L.x1.z - L.x0.z};
     const float e2[3] = {L.x2.x - L.x0.x, L.x2.y - L.x0.y, L.x2.z - L.x0.z};
@@ -126,9 +141,13 @@ __device__ __forceinline__ void local_corners(const LocalIn& L, float (&out)[4][
         for (int j = 0; j < 3; ++j) F[i][j] = e1[i] * g1[j] + e2[i] * g2[j] + e3[i] * g3[j];
     float P[3][3];
     const float ws = L.r1.w, wv = L.r2.w;
-    Strain S;
-    if (strain_of<false>(F, S)) strain_apply<RESID>(F, S, ws, wv, P);
-    else svd_apply<RESID>(F, ws, wv, P);
+    if (FAST) {
+        Strain S;
+        if (strain_of<false>(F, S)) strain_apply<RESID>(F, S, ws, wv, P);
+        else svd_targets_rare<RESID>(F, ws, wv, P);
+    } else {
+        svd_targets<RESID>(F, ws, wv, P);
+    }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         out[1][i] = P[i][0] * g1[0] + P[i][1] * g1[1] + P[i][2] * g1[2];
@@ -164,7 +183,7 @@ __device__ __forceinline__ float4 assembly_base(const LocalAsmArgs& A, int v) {
 }
 
 // One block of the fused kernel: tets [blk kLaTets, (blk + 1) kLaTets) of the mesh in A.
-template <bool RESID>
+template <bool RESID, bool FAST>
 __device__ __forceinline__ void local_assemble_block(const LocalAsmArgs& A, int blk) {
     __shared__ float fx[4 * kLaTets], fy[4 * kLaTets], fz[4 * kLaTets];
     pdl_trigger();
@@ -183,7 +202,7 @@ __device__ __forceinline__ void local_assemble_block(const LocalAsmArgs& A, int 
     L.x2 = A.x[tv.z];
     L.x3 = A.x[tv.w];
     float f[4][3];
-    local_corners<RESID>(L, f);
+    local_corners<RESID, FAST>(L, f);
     if (live) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -213,9 +232,9 @@ __device__ __forceinline__ void local_assemble_block(const LocalAsmArgs& A, int 
     }
 }
 
-template <bool RESID>
+template <bool RESID, bool FAST>
 __global__ void __launch_bounds__(kLaTets, PDG_LA_MINB) k_local_assemble(LocalAsmArgs A) {
-    local_assemble_block<RESID>(A, blockIdx.x);
+    local_assemble_block<RESID, FAST>(A, blockIdx.x);
 }
 
 // shared vertices: b_v = base + the blocks' partial sums in block order
@@ -268,7 +287,7 @@ __device__ __forceinline__ LocalAsmArgs batch_args(const BatchSlot& S) {
 __global__ void __launch_bounds__(kLaTets, PDG_LA_MINB) k_b_local_assemble(const BatchSlot* __restrict__ slots,
                                                                          const int* __restrict__ off, int n_slots) {
     const int s = batch_find_slot(off, n_slots, blockIdx.x);
-    local_assemble_block<false>(batch_args(slots[s]), blockIdx.x - off[s]);
+    local_assemble_block<false, true>(batch_args(slots[s]), blockIdx.x - off[s]);
 }
 
 __global__ void __launch_bounds__(256) k_b_assemble_shared(const BatchSlot* __restrict__ slots,
@@ -360,7 +379,7 @@ void build_local_plan(pd_mesh* m, const std::vector<int32_t>& inc_ptr, const std
 }
 
 void launch_local_assemble(const pd_mesh* m, const float4* x, const float4* by0, const float4* y, float4* b,
-                           bool residual, cudaStream_t s) {
+                           bool residual, bool fast, cudaStream_t s) {
     if (m->n_t <= 0) return;
     LocalAsmArgs A{};
     A.n_t = m->n_t;
@@ -380,12 +399,13 @@ void launch_local_assemble(const pd_mesh* m, const float4* x, const float4* by0,
     A.sh_vert = m->d_la_sh_vert.p;
     A.part = m->d_la_part.p;
     const int nsb = (m->la_shared + 255) / 256;
-    if (residual) {
-        launch_pdl(k_local_assemble<true>, dim3(m->la_blocks), dim3(kLaTets), 0, s, A);
-        if (nsb > 0) launch_pdl(k_assemble_shared<true>, dim3(nsb), dim3(256), 0, s, A, m->la_shared);
-    } else {
-        launch_pdl(k_local_assemble<false>, dim3(m->la_blocks), dim3(kLaTets), 0, s, A);
-        if (nsb > 0) launch_pdl(k_assemble_shared<false>, dim3(nsb), dim3(256), 0, s, A, m->la_shared);
+    const dim3 grid(m->la_blocks), block(kLaTets);
+    if (residual) launch_pdl(k_local_assemble<true, true>, grid, block, 0, s, A);
+    else if (fast) launch_pdl(k_local_assemble<false, true>, grid, block, 0, s, A);
+    else launch_pdl(k_local_assemble<false, false>, grid, block, 0, s, A);
+    if (nsb > 0) {
+        if (residual) launch_pdl(k_assemble_shared<true>, dim3(nsb), dim3(256), 0, s, A, m->la_shared);
+        else launch_pdl(k_assemble_shared<false>, dim3(nsb), dim3(256), 0, s, A, m->la_shared);
     }
     PDG_CHECK_LAUNCH();
 }

@@ -1675,7 +1675,7 @@ static void run_frame(pd_mesh* m, int n_iter, const float g[3], cudaStream_t s) 
         // fused local step and assembly: the RHS b, or in the correction form
         // the residual b - K x itself (formed per tet without cancellation)
         phase_begin(m, PH_LOCAL, s);
-        launch_local_assemble(m, m->d_x.p, m->d_by0.p, m->d_y.p, m->d_b.p, m->correction, s);
+        launch_local_assemble(m, m->d_x.p, m->d_by0.p, m->d_y.p, m->d_b.p, m->correction, m->correction, s);
         phase_end(m, s);
         if (m->correction) {
             launch_dd_solve(m, m->d_b.p, m->d_dx.p, s, false);
@@ -1863,7 +1863,7 @@ pd_status pd_local_rhs(pd_mesh* m, const float* x, const float* y, float* b) {
         PDG_CUDA(cudaMemcpyAsync(m->d_pin_tgt.p, xi.p + m->n_free, sizeof(float4) * m->n_pin,
                                  cudaMemcpyDeviceToDevice, s));
     launch_by0_from_y(m, yi.p, by0.p, s);
-    launch_local_assemble(m, xi.p, by0.p, nullptr, bb.p, false, s);
+    launch_local_assemble(m, xi.p, by0.p, nullptr, bb.p, false, true, s);
     launch_scatter_out(m, bb.p, b, 1, s);
     PDG_CUDA(cudaStreamSynchronize(s));
     return PD_OK;

@@ -601,9 +601,10 @@ void jacobi_eig(std::vector<double>& A, int q, std::vector<double>& w, std::vect
 void launch_project(const float* F, int n, float* R, float* V, float* sig, cudaStream_t s);
 void build_local_plan(pd_mesh* m, const std::vector<int32_t>& inc_ptr, const std::vector<int32_t>& inc,
                       cudaStream_t s);
-// fused local step + assembly: b = by0 + sum (RHS form) or b = (M/dt^2)(y - x) + sum (residual form)
+// fused local step + assembly: b = by0 + sum (RHS form) or b = (M/dt^2)(y - x) + sum (residual form, always SVD-free);
+// fast: the SVD-free targets in the RHS form
 void launch_local_assemble(const pd_mesh* m, const float4* x, const float4* by0, const float4* y, float4* b,
-                           bool residual, cudaStream_t s);
+                           bool residual, bool fast, cudaStream_t s);
 void launch_inertia(const pd_mesh* m, float h, float gx, float gy, float gz, cudaStream_t s);
 void launch_velocity(const pd_mesh* m, float inv_h, cudaStream_t s);
 void launch_pin_copy(const pd_mesh* m, const float* user_targets, cudaStream_t s);
