@@ -56,10 +56,12 @@ __global__ void k_b_inertia(const BatchSlot* __restrict__ slots, const int* __re
 }
 
 __global__ void k_b_gather(const BatchSlot* __restrict__ slots, const int* __restrict__ off, int n_slots) {
+    pdl_trigger();
     const int s = batch_find_slot(off, n_slots, blockIdx.x);
     const BatchSlot& S = slots[s];
     const int j = (blockIdx.x - off[s]) * blockDim.x + threadIdx.x;
     if (j >= S.n_B) return;
+    pdl_wait();
     float4 acc = S.b[S.n_int + j];
     for (int k = S.gat_ptr[j]; k < S.gat_ptr[j + 1]; ++k) {
         const float4 c = S.tc[S.gat[k]];
@@ -70,10 +72,12 @@ __global__ void k_b_gather(const BatchSlot* __restrict__ slots, const int* __res
 
 // two-level requests: c_T = c_B[T0:] + the gathered second-level terms (as k_gather)
 __global__ void k_b_gather2(const BatchSlot* __restrict__ slots, const int* __restrict__ off, int n_slots) {
+    pdl_trigger();
     const int s = batch_find_slot(off, n_slots, blockIdx.x);
     const BatchSlot& S = slots[s];
     const int j = (blockIdx.x - off[s]) * blockDim.x + threadIdx.x;
     if (j >= S.n_top) return;
+    pdl_wait();
     float4 acc = S.cB[S.n_B - S.n_top + j];
     for (int k = S.gat2_ptr[j]; k < S.gat2_ptr[j + 1]; ++k) {
         const float4 c = S.tc2[S.gat2[k]];
@@ -83,10 +87,12 @@ __global__ void k_b_gather2(const BatchSlot* __restrict__ slots, const int* __re
 }
 
 __global__ void k_b_reduce(const BatchSlot* __restrict__ slots, const int* __restrict__ off, int n_slots) {
+    pdl_trigger();
     const int s = batch_find_slot(off, n_slots, blockIdx.x);
     const BatchSlot& S = slots[s];
     const int j = (blockIdx.x - off[s]) * blockDim.x + threadIdx.x;
     if (j >= S.n_B) return;
+    pdl_wait();
     float4 acc = S.part[j];
     for (int c = 1; c < S.nch; ++c) {
         const float4 p = S.part[(int64_t)c * S.n_B + j];
@@ -128,17 +134,17 @@ void launch_b_inertia(const BatchSlot* slots, const int* off, int n_slots, int b
 }
 void launch_b_gather(const BatchSlot* slots, const int* off, int n_slots, int blocks, cudaStream_t s) {
     if (blocks <= 0) return;
-    k_b_gather<<<blocks, 256, 0, s>>>(slots, off, n_slots);
+    launch_pdl(k_b_gather, dim3(blocks), dim3(256), 0, s, slots, off, n_slots);
     PDG_CHECK_LAUNCH();
 }
 void launch_b_gather2(const BatchSlot* slots, const int* off, int n_slots, int blocks, cudaStream_t s) {
     if (blocks <= 0) return;
-    k_b_gather2<<<blocks, 256, 0, s>>>(slots, off, n_slots);
+    launch_pdl(k_b_gather2, dim3(blocks), dim3(256), 0, s, slots, off, n_slots);
     PDG_CHECK_LAUNCH();
 }
 void launch_b_reduce(const BatchSlot* slots, const int* off, int n_slots, int blocks, cudaStream_t s) {
     if (blocks <= 0) return;
-    k_b_reduce<<<blocks, 256, 0, s>>>(slots, off, n_slots);
+    launch_pdl(k_b_reduce, dim3(blocks), dim3(256), 0, s, slots, off, n_slots);
     PDG_CHECK_LAUNCH();
 }
 void launch_b_velocity(const BatchSlot* slots, const int* off, int n_slots, int blocks, cudaStream_t s) {

@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(32 * (kAxtWarps + 1)) k_axpy_tma(const AxDesc*
     const T* tile = reinterpret_cast<const T*>(B.pool) + D.a_off + (int64_t)bk.o0 * D.K;
     const int n_st = (D.K + R - 1) / R;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    pdl_trigger();
+    if (!single.late) pdl_trigger();
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < S; ++k) {
@@ -445,7 +445,8 @@ __global__ void __launch_bounds__(32 * (kAxtWarps + 1)) k_axpy_tma(const AxDesc*
                 if (blockIdx.x == 0 && i == 0 && *reinterpret_cast<volatile int*>(&g_test_copy_extra) > 0)
                     expect += (uint32_t)max(atomicExch(&g_test_copy_extra, 0), 0);
                 mbar_arrive_expect_tx(&full[slot], expect);
-                bulk_g2s(ring + (size_t)slot * R * w, tile + (int64_t)i * R * w, bytes, &full[slot]);
+                if (single.once) bulk_g2s_once(ring + (size_t)slot * R * w, tile + (int64_t)i * R * w, bytes, &full[slot]);
+                else bulk_g2s(ring + (size_t)slot * R * w, tile + (int64_t)i * R * w, bytes, &full[slot]);
                 issued = i + 1;
             }
             // every copy issued has landed before the CTA may exit
@@ -616,7 +617,7 @@ __global__ void __launch_bounds__(32 * (kAxtWarps + 1)) k_axpy_mma(const AxDesc*
     const E* tile = reinterpret_cast<const E*>(B.pool) + D.a_off + (int64_t)bk.o0 * Kp;
     const int n_st = (Kp + R - 1) / R;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    pdl_trigger();
+    if (!B.late) pdl_trigger();
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < S; ++k) {
@@ -645,7 +646,8 @@ __global__ void __launch_bounds__(32 * (kAxtWarps + 1)) k_axpy_mma(const AxDesc*
                 if (blockIdx.x == 0 && i == 0 && *reinterpret_cast<volatile int*>(&g_test_copy_extra) > 0)
                     expect += (uint32_t)max(atomicExch(&g_test_copy_extra, 0), 0);
                 mbar_arrive_expect_tx(&full[slot], expect);
-                bulk_g2s(ring + (size_t)slot * R * w, tile + (int64_t)i * R * w, bytes, &full[slot]);
+                if (B.once) bulk_g2s_once(ring + (size_t)slot * R * w, tile + (int64_t)i * R * w, bytes, &full[slot]);
+                else bulk_g2s(ring + (size_t)slot * R * w, tile + (int64_t)i * R * w, bytes, &full[slot]);
                 issued = i + 1;
             }
             for (int i = max(0, issued - S); i < issued; ++i)
@@ -916,6 +918,7 @@ __global__ void __launch_bounds__(512, 1) k_coarse_b(const CoarseDescB* __restri
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int64_t b0 = U * blockIdx.x / gridDim.x, b1 = U * (blockIdx.x + 1) / gridDim.x;
+    pdl_wait();   // c_B comes from the predecessor (the successor starts when this kernel ends)
     for (int di = 0; di < n_desc; ++di) {
         const CoarseDescB D = cd[di];
         const int64_t nu = (int64_t)((D.n_B + 1) / 2) * D.nch;
@@ -1106,6 +1109,8 @@ __global__ void k_residual(int n_free, const int* __restrict__ ptr, const int* _
 }
 
 __global__ void k_axpy(int n, const float4* __restrict__ dx, float4* __restrict__ x) {
+    pdl_trigger();
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     float4 a = x[i], d = dx[i];
@@ -1181,7 +1186,7 @@ __global__ void __launch_bounds__(32 * (kRowtWarps + 1)) k_rowdot_tma(const RowD
     const int warp = threadIdx.x >> 5;
     const int64_t b0 = blk_u[blockIdx.x], b1 = blk_u[blockIdx.x + 1];
     const T* pool = reinterpret_cast<const T*>(B.pool);
-    pdl_trigger();
+    if (!B.late) pdl_trigger();
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < S; ++k) {
@@ -1218,7 +1223,8 @@ __global__ void __launch_bounds__(32 * (kRowtWarps + 1)) k_rowdot_tma(const RowD
                     const uint32_t bytes = (uint32_t)rows * (uint32_t)D.ld * (uint32_t)sizeof(T);
                     mbar_arrive_expect_tx(&full[slot], bytes);
                     const T* pl = BATCHED ? reinterpret_cast<const T*>(multi[D.slot].pool) : pool;
-                    bulk_g2s(ring + (size_t)slot * SE, pl + D.a_off + (int64_t)r * D.ld, bytes, &full[slot]);
+                    if (B.once) bulk_g2s_once(ring + (size_t)slot * SE, pl + D.a_off + (int64_t)r * D.ld, bytes, &full[slot]);
+                    else bulk_g2s(ring + (size_t)slot * SE, pl + D.a_off + (int64_t)r * D.ld, bytes, &full[slot]);
                     issued = g + 1;
                 }
             }
@@ -1360,7 +1366,7 @@ __global__ void __launch_bounds__(32 * (kRowtWarps + 1)) k_rowdot_mma(const RowD
     const int warp = threadIdx.x >> 5;
     const int64_t b0 = blk_u[blockIdx.x], b1 = blk_u[blockIdx.x + 1];
     const __nv_bfloat16* pool = reinterpret_cast<const __nv_bfloat16*>(B.pool);
-    pdl_trigger();
+    if (!B.late) pdl_trigger();
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < S; ++k) {
@@ -1395,7 +1401,8 @@ __global__ void __launch_bounds__(32 * (kRowtWarps + 1)) k_rowdot_mma(const RowD
                         }
                         const uint32_t bytes = (uint32_t)min(SB, nkb - kb0) * 512u;
                         mbar_arrive_expect_tx(&full[slot], bytes);
-                        bulk_g2s(ring + (size_t)slot * (SB * 256), row + (int64_t)kb0 * 256, bytes, &full[slot]);
+                        if (B.once) bulk_g2s_once(ring + (size_t)slot * (SB * 256), row + (int64_t)kb0 * 256, bytes, &full[slot]);
+                        else bulk_g2s(ring + (size_t)slot * (SB * 256), row + (int64_t)kb0 * 256, bytes, &full[slot]);
                         issued = g + 1;
                     }
                 }
@@ -1565,15 +1572,22 @@ void launch_ax(const AxDesc* descs, const AxBlock* blocks, int n_blocks, int k_m
 }
 
 template <class T>
-void launch_rowdot(const RowPlan& P, const AxBases& B, cudaStream_t s, int* tma_err = nullptr) {
+void launch_rowdot(const RowPlan& P, const AxBases& B, cudaStream_t s, int* tma_err = nullptr, bool pdl = false) {
     if (P.n_blocks <= 0) return;
+    const dim3 grid(P.n_blocks), block(32 * (kRowtWarps + 1));
+    const RowDesc* descs = P.descs.p;
+    const int64_t* units = P.blk_u.p;
     if (P.mma && tma_err) {
-        k_rowdot_mma<<<P.n_blocks, 32 * (kRowtWarps + 1), rowm_smem_bytes(P.xcap), s>>>(P.descs.p, P.n_desc, P.blk_u.p,
-                                                                                     B, P.xcap, tma_err);
+        const size_t smem = rowm_smem_bytes(P.xcap);
+        if (pdl) launch_pdl(k_rowdot_mma, grid, block, smem, s, descs, P.n_desc, units, B, P.xcap, tma_err);
+        else k_rowdot_mma<<<grid, block, smem, s>>>(descs, P.n_desc, units, B, P.xcap, tma_err);
     } else if (P.tma && tma_err) {
         const size_t smem = (size_t)kRowtStages * kRowtStageBytes + sizeof(float) * 3 * (size_t)P.xcap;
-        k_rowdot_tma<T, false><<<P.n_blocks, 32 * (kRowtWarps + 1), smem, s>>>(P.descs.p, P.n_desc, P.blk_u.p, B,
-                                                                              nullptr, P.xcap, tma_err);
+        if (pdl)
+            launch_pdl(k_rowdot_tma<T, false>, grid, block, smem, s, descs, P.n_desc, units, B, (const AxBases*)nullptr,
+                       P.xcap, tma_err);
+        else
+            k_rowdot_tma<T, false><<<grid, block, smem, s>>>(descs, P.n_desc, units, B, nullptr, P.xcap, tma_err);
     } else {
         k_rowdot<T><<<P.n_blocks, 32 * kRowWarps, sizeof(float) * 3 * (size_t)P.xcap, s>>>(P.descs.p, P.n_desc,
                                                                                              P.blk_u.p, B, P.xcap);
@@ -1621,11 +1635,30 @@ void dd_solve_stream(pd_mesh* m, const float4* b, float4* xout, const DDBufs& w,
     phase_end(m, s);
 }
 
+// One product's arrays and launch properties.
+//   once: the per-domain matrices and S_II^-1 are most of an iteration's bytes (253 of 398 MB on the 390K shell, FP32)
+//     and return only in the next iteration; leaving L2 first, they keep the interface chain's matrices in it (129
+//     MB).  Frames measured without / with: 140K-tet shell FP32 1.07 / 0.94 ms, 390K BF16 1.65 / 1.59, 390K FP32 2.00 /
+//     1.98; no difference where everything fits (53K-tet shell).
+//   late: see dd_solve_impl.
+AxBases product(const void* pool, const float4* x, const int* bidx, const float4* add, float4* out, bool once, bool late) {
+    AxBases B{pool, x, bidx, add, out};
+    B.once = once;
+    B.late = late;
+    return B;
+}
+
 template <class T>
 void dd_solve_impl(pd_mesh* m, const T* pool, const float4* b, float4* xout, const DDBufs& w, cudaStream_t s) {
     // the interior part t = K_ii^-1 b_i runs on a side stream beside the
     // interface solve and is joined before the back-substitution
     const bool fork1 = m->ax_blocks_int > 0 || m->ax_blocks_m1 > 0;
+    // One interface level: the coarse product is a programmatic launch too, but neither it nor the condensation
+    // lets its successor start early: a coarse block holds 90 KB of shared memory, and blocks waiting for their
+    // turn keep the running ones (and the interior product's) from the SMs.  20 iterations measured with the
+    // successors started early / so: 53K-tet shell TF32 676 / 601 us, FP32 550 / 495, 12K slab 477 / 444.  (Two levels:
+    // the early start of the gather after the condensation gains 1.5 % in FP32, the row-form products are plain launches.)
+    const bool direct = !m->two_level;
     if (fork1) {
         PDG_CUDA(cudaEventRecord(m->ev_fork[0], s));
         PDG_CUDA(cudaStreamWaitEvent(m->side[0], m->ev_fork[0], 0));
@@ -1646,7 +1679,7 @@ void dd_solve_impl(pd_mesh* m, const T* pool, const float4* b, float4* xout, con
             for (int b0 = 0; b0 < nb; b0 += per) {
                 phase_begin(m, PH_INTERIOR, m->side[0]);   // (timed per launch)
                 launch_ax<T>(m->d_ax_desc_int.p, m->d_ax_blk_int.p + b0, std::min(per, nb - b0), m->ax_kmax_int,
-                             AxBases{pool, b, nullptr, nullptr, w.tc}, m->side[0], m->ax_tiled ? m->d_err.p : nullptr,
+                             product(pool, b, nullptr, nullptr, w.tc, true, false), m->side[0], m->ax_tiled ? m->d_err.p : nullptr,
                              m->ax_wmax_int, false, m->ax_tf32);
                 phase_end(m, m->side[0]);
             }
@@ -1656,7 +1689,7 @@ void dd_solve_impl(pd_mesh* m, const T* pool, const float4* b, float4* xout, con
     if (m->ax_blocks_cond > 0) {
         phase_begin(m, PH_CONDENSE, s);
         launch_ax<T>(m->d_ax_desc_cond.p, m->d_ax_blk_cond.p, m->ax_blocks_cond, m->ax_kmax_cond,
-                     AxBases{pool, b, nullptr, nullptr, w.tc}, s, m->ax_tiled ? m->d_err.p : nullptr, m->ax_wmax_cond,
+                     product(pool, b, nullptr, nullptr, w.tc, true, direct), s, m->ax_tiled ? m->d_err.p : nullptr, m->ax_wmax_cond,
                      true, m->ax_tf32);
         phase_end(m, s);
     }
@@ -1676,7 +1709,7 @@ void dd_solve_impl(pd_mesh* m, const T* pool, const float4* b, float4* xout, con
                 PDG_CUDA(cudaEventRecord(m->ev_fork[1], s));
                 PDG_CUDA(cudaStreamWaitEvent(m->side[1], m->ev_fork[1], 0));
                 phase_begin(m, PH_INTERIOR2, m->side[1]);
-                launch_rowdot<T>(m->rows_int2, AxBases{pool, w.cB, nullptr, nullptr, w.tc2}, m->side[1], m->d_err.p);
+                launch_rowdot<T>(m->rows_int2, product(pool, w.cB, nullptr, nullptr, w.tc2, true, false), m->side[1], m->d_err.p);
                 phase_end(m, m->side[1]);
                 PDG_CUDA(cudaEventRecord(m->ev_join[1], m->side[1]));
             }
@@ -1694,7 +1727,7 @@ void dd_solve_impl(pd_mesh* m, const T* pool, const float4* b, float4* xout, con
         if (m->rows_coarse.n_blocks > 0) {
             // BF16 on the tensor cores: whole block-rows, written straight to x
             phase_begin(m, PH_COARSE, s);
-            launch_rowdot<T>(m->rows_coarse, AxBases{pool, cin, nullptr, nullptr, xcs}, s, m->d_err.p);
+            launch_rowdot<T>(m->rows_coarse, product(pool, cin, nullptr, nullptr, xcs, false, direct), s, m->d_err.p, direct);
             phase_end(m, s);
         } else {
             phase_begin(m, PH_COARSE, s);
@@ -1718,7 +1751,7 @@ void dd_solve_impl(pd_mesh* m, const T* pool, const float4* b, float4* xout, con
     if (m->ax_blocks_back > 0) {
         phase_begin(m, PH_BACKSUB, s);
         launch_ax<T>(m->d_ax_desc_back.p, m->d_ax_blk_back.p, m->ax_blocks_back, m->ax_kmax_back,
-                     AxBases{pool, xout + m->n_int, m->d_bidx.p, w.tc, xout}, s, m->ax_tiled ? m->d_err.p : nullptr,
+                     product(pool, xout + m->n_int, m->d_bidx.p, w.tc, xout, true, false), s, m->ax_tiled ? m->d_err.p : nullptr,
                      m->ax_wmax_back, true, m->ax_tf32);
         phase_end(m, s);
     }
@@ -1758,13 +1791,15 @@ void launch_dd_solve_scratch(pd_mesh* m, const float4* b, float4* xout, float4* 
 // Serving batches: every resident request's tiled products in one launch of
 // the bulk-copy kernel (each block reads its request's arrays from `bases`).
 void launch_axpy_b(const AxDesc* descs, const AxBlock* blocks, const AxBases* bases, int n_blocks, int k_max,
-                   int w_max, int* err, cudaStream_t s) {
+                   int w_max, int* err, bool late, cudaStream_t s) {
     if (n_blocks <= 0) return;
     const size_t ring = axt_ring_bytes<float>(w_max);
     const size_t smem = ring + sizeof(float4) * std::max(k_max, 1);
     if ((int)smem > axt_smem_limit<float>()) throw Fail{PD_ERR_UNSUPPORTED};
-    k_axpy_tma<float, true><<<n_blocks, 32 * (kAxtWarps + 1), smem, s>>>(descs, blocks, AxBases{}, bases, (int)ring,
-                                                                          err);
+    AxBases launch{};
+    launch.late = late;
+    launch_pdl(k_axpy_tma<float, true>, dim3(n_blocks), dim3(32 * (kAxtWarps + 1)), smem, s, descs, blocks, launch, bases,
+               (int)ring, err);
     PDG_CHECK_LAUNCH();
 }
 
@@ -1798,7 +1833,8 @@ bool configure_coarse_b(int max_cols) {
 
 void launch_coarse_b(const CoarseDescB* cd, int n_desc, int64_t U, int max_cols, int blocks, cudaStream_t s) {
     if (blocks <= 0 || U <= 0) return;
-    k_coarse_b<<<blocks, 32 * kCoarseWarps, sizeof(float) * 3 * (size_t)max_cols, s>>>(cd, n_desc, U, max_cols);
+    launch_pdl(k_coarse_b, dim3(blocks), dim3(32 * kCoarseWarps), sizeof(float) * 3 * (size_t)max_cols, s, cd, n_desc, U,
+               max_cols);
     PDG_CHECK_LAUNCH();
 }
 
@@ -1930,7 +1966,7 @@ void launch_residual(const pd_mesh* m, const float4* b, const float4* x, float4*
 
 void launch_axpy_free(const pd_mesh* m, const float4* dx, float4* x, cudaStream_t s) {
     if (m->n_free <= 0) return;
-    k_axpy<<<nblk(m->n_free, 256), 256, 0, s>>>(m->n_free, dx, x);
+    launch_pdl(k_axpy, dim3(nblk(m->n_free, 256)), dim3(256), 0, s, m->n_free, dx, x);
     PDG_CHECK_LAUNCH();
 }
 

@@ -412,13 +412,13 @@ void launch_local_assemble(const pd_mesh* m, const float4* x, const float4* by0,
 
 void launch_b_local_assemble(const BatchSlot* slots, const int* off, int n_slots, int blocks, cudaStream_t s) {
     if (blocks <= 0) return;
-    k_b_local_assemble<<<blocks, kLaTets, 0, s>>>(slots, off, n_slots);
+    launch_pdl(k_b_local_assemble, dim3(blocks), dim3(kLaTets), 0, s, slots, off, n_slots);
     PDG_CHECK_LAUNCH();
 }
 
 void launch_b_assemble_shared(const BatchSlot* slots, const int* off, int n_slots, int blocks, cudaStream_t s) {
     if (blocks <= 0) return;
-    k_b_assemble_shared<<<blocks, 256, 0, s>>>(slots, off, n_slots);
+    launch_pdl(k_b_assemble_shared, dim3(blocks), dim3(256), 0, s, slots, off, n_slots);
     PDG_CHECK_LAUNCH();
 }
 

@@ -156,6 +156,9 @@ struct AxBases {
     const int* bidx;       // gather list (boundary products) or null
     const float4* add;     // added to the result, or null
     float4* out;
+    // of the launch (a batched one reads them from `single`, not from its slots):
+    bool once = false;     // the matrix leaves L2 first (see launch_products in k_dd.cu)
+    bool late = false;     // the next kernel of the chain is not started before this one ends
 };
 struct AxDesc {
     int64_t a_off;         // pool offset of row 0

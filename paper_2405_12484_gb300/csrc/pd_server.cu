@@ -35,7 +35,7 @@ void launch_rowdot_b(const RowPlan& P, const AxBases* multi, int* err, cudaStrea
 void build_row_plan(RowPlan& P, std::vector<RowDesc> descs, int prec, cudaStream_t s, bool mma);
 void launch_b_velocity(const BatchSlot* slots, const int* off, int n_slots, int blocks, cudaStream_t s);
 void launch_axpy_b(const AxDesc* descs, const AxBlock* blocks, const AxBases* bases, int n_blocks, int k_max,
-                   int w_max, int* err, cudaStream_t s);
+                   int w_max, int* err, bool late, cudaStream_t s);
 int ax_outputs_per_block(int prec);
 bool configure_coarse_b(int max_cols);
 void launch_coarse_b(const CoarseDescB* cd, int n_desc, int64_t U, int max_cols, int blocks, cudaStream_t s);
@@ -365,7 +365,7 @@ static void rebuild(pd_server* S) {
         for (int it = 0; it < S->n_iter; ++it) {
             launch_b_local_assemble(sl, S->d_off[PH_LOC].p, n, S->blocks[PH_LOC], c);
             launch_b_assemble_shared(sl, S->d_off[PH_ASM].p, n, S->blocks[PH_ASM], c);
-            launch_axpy_b(S->d_axc.p, S->d_blkc.p, S->d_basc.p, S->blocks_c, S->kmax_c, S->wmax_c, S->d_err.p, c);
+            launch_axpy_b(S->d_axc.p, S->d_blkc.p, S->d_basc.p, S->blocks_c, S->kmax_c, S->wmax_c, S->d_err.p, true, c);
             launch_b_gather(sl, S->d_off[PH_GAT].p, n, S->blocks[PH_GAT], c);
             launch_rowdot_b(S->rows_r2, S->d_basr2.p, S->d_err.p, c);
             launch_b_gather2(sl, S->d_off[PH_GAT2].p, n, S->blocks[PH_GAT2], c);
@@ -373,7 +373,7 @@ static void rebuild(pd_server* S) {
             launch_rowdot_b(S->rows_co, S->d_basco.p, S->d_err.p, c);
             launch_b_reduce(sl, S->d_off[PH_RED].p, n, S->blocks[PH_RED], c);
             launch_rowdot_b(S->rows_b2, S->d_basb2.p, S->d_err.p, c);
-            launch_axpy_b(S->d_axb.p, S->d_blkb.p, S->d_basb.p, S->blocks_b, S->kmax_b, S->wmax_b, S->d_err.p, c);
+            launch_axpy_b(S->d_axb.p, S->d_blkb.p, S->d_basb.p, S->blocks_b, S->kmax_b, S->wmax_b, S->d_err.p, false, c);
         }
         launch_b_velocity(sl, S->d_off[PH_VEL].p, n, S->blocks[PH_VEL], c);
     } catch (...) {

@@ -71,5 +71,17 @@ static __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint
         : "memory");
 }
 
+// The same copy for bytes that the next pass over the data will not find in L2 anyway: they leave it first, so
+// that what fits stays.
+static __device__ __forceinline__ void bulk_g2s_once(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    uint64_t policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
+            smem_u32(dst)),
+        "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
+        : "memory");
+}
+
 }  // namespace tma
 }  // namespace pdg
