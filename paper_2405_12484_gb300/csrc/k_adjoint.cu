@@ -4,7 +4,7 @@
 //  * k_grad_local / k_assemble_residual: g = (M/dt^2)(x - y) + grad E(x),
 //    the equilibrium residual of Eq. g, with per-tet contributions
 //    (ws (F - R) + wv (F - V)) g_c = U diag(ws (s - 1) + wv (s - d)) W^T g_c;
-//  * k_hvp_local / k_assemble_hvp: H v = (M/dt^2) v + sum_e d^2E_e[v], with
+//  * H v = (M/dt^2) v + sum_e d^2E_e[v] (k_hvp_local / k_assemble_hvp, and k_hvp_terms / k_pcg_hvp inside the CG), with
 //    d^2E_e/dF^2 = V_e [gs (I - dR/dF) + gv (I - dV/dF)] from the derivative
 //    of an isotropic matrix function P = U diag(f(s)) W^T:  A = U^T dF W,
 //    (U^T dP W)_ii = sum_k (df_i/ds_k) A_kk and, for i != j,
@@ -12,7 +12,7 @@
 //    alpha_ij = (f_i - f_j)/(s_i - s_j), beta_ij = (f_i + f_j)/(s_i + s_j);
 //  * k_grad_gamma: dL/dgamma_e -= V_e <F - R, Lambda_e> (and <F - V, .>),
 //    Lambda_e = sum_c lambda_c (outer) g_c (the adjoint's own gradient);
-//  * deterministic FP64 dot products and the PCG vector updates.
+//  * deterministic FP64 dot products and the preconditioned CG iteration.
 #include <algorithm>
 
 #include "pd_internal.h"
@@ -104,74 +104,298 @@ __device__ __forceinline__ void volume_jacobian(const float (&s)[3], const float
         for (int k = 0; k < 3; ++k) J[i][k] = (fr[i] && fr[k]) ? ((i == k ? a[i] * d[i] : 0.f) - a[i] * a[k] * iS) : 0.f;
 }
 
+// d^2E_e in the singular frame of F, weights included: B_ii = sum_k J_ik A_kk, B_ij = al_ij sym_ij + be_ij skw_ij, and
+// dP = (ws + wv) dF - U B W^T.  Thirty floats (U, W, J and the pairs 01, 02, 12), constant over a linear solve.
+struct Hess {
+    float U[3][3], W[3][3];
+    float J[6];           // 00 01 02 11 12 22
+    float al[3], be[3];   // pairs 01 02 12
+};
+constexpr int kHessFloats = 30;
+
+__device__ __forceinline__ void hess_terms(const Tet& T, const float (&F)[3][3], Hess& H) {
+    float s[3], d[3], J[3][3], sq[3];
+    bool fr[3];
+    svd3(F, H.U, s, H.W);
+    volume_targets(s, d);
+    volume_jacobian(s, d, J, fr, sq);
+    H.J[0] = T.wv * J[0][0];
+    H.J[1] = T.wv * J[0][1];
+    H.J[2] = T.wv * J[0][2];
+    H.J[3] = T.wv * J[1][1];
+    H.J[4] = T.wv * J[1][2];
+    H.J[5] = T.wv * J[2][2];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const int i = q == 2 ? 1 : 0, j = q == 0 ? 1 : 2;
+        float ssum = s[i] + s[j];
+        if (fabsf(ssum) < 1e-6f) ssum = copysignf(1e-6f, ssum);
+        const float betaR = 2.f / ssum;
+        const float betaV = (d[i] + d[j]) / ssum;
+        float alphaV;
+        if (fr[i] && fr[j] && sq[i] > 0.f && sq[j] > 0.f) {
+            // both on the + branch: (d_i - d_j)/(s_i - s_j) without cancellation
+            alphaV = 0.5f * (1.f + (s[i] + s[j]) / (sq[i] + sq[j]));
+        } else if (fabsf(s[i] - s[j]) > 1e-6f * fmaxf(1.f, fabsf(s[i]))) {
+            alphaV = (d[i] - d[j]) / (s[i] - s[j]);
+        } else {
+            alphaV = J[i][i] - J[i][j];
+        }
+        H.al[q] = T.wv * alphaV;
+        H.be[q] = T.ws * betaR + T.wv * betaV;
+    }
+}
+
+__device__ __forceinline__ void hess_apply(const Hess& H, float wsum, const float (&dF)[3][3], float (&dP)[3][3]) {
+    // A = U^T dF W
+    float A[3][3], T1[3][3], B[3][3], UB[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) T1[i][j] = dF[i][0] * H.W[0][j] + dF[i][1] * H.W[1][j] + dF[i][2] * H.W[2][j];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) A[i][j] = H.U[0][i] * T1[0][j] + H.U[1][i] * T1[1][j] + H.U[2][i] * T1[2][j];
+    B[0][0] = H.J[0] * A[0][0] + H.J[1] * A[1][1] + H.J[2] * A[2][2];
+    B[1][1] = H.J[1] * A[0][0] + H.J[3] * A[1][1] + H.J[4] * A[2][2];
+    B[2][2] = H.J[2] * A[0][0] + H.J[4] * A[1][1] + H.J[5] * A[2][2];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const int i = q == 2 ? 1 : 0, j = q == 0 ? 1 : 2;
+        const float sym = 0.5f * H.al[q] * (A[i][j] + A[j][i]), skw = 0.5f * H.be[q] * (A[i][j] - A[j][i]);
+        B[i][j] = sym + skw;
+        B[j][i] = sym - skw;
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) UB[i][j] = H.U[i][0] * B[0][j] + H.U[i][1] * B[1][j] + H.U[i][2] * B[2][j];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            dP[i][j] = wsum * dF[i][j] - (UB[i][0] * H.W[j][0] + UB[i][1] * H.W[j][1] + UB[i][2] * H.W[j][2]);
+}
+
 __global__ void __launch_bounds__(128) k_hvp_local(int n_t, const int4* __restrict__ tets,
                                                    const float4* __restrict__ geo, const float4* __restrict__ x,
                                                    const float4* __restrict__ v, float4* __restrict__ force) {
     int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n_t) return;
     const Tet T = load_tet(e, n_t, tets, geo);
-    float F[3][3], U[3][3], W[3][3], s[3], d[3], dF[3][3];
+    float F[3][3], dF[3][3], dP[3][3];
     tet_grad(T, x, F);
     tet_grad(T, v, dF);
-    svd3(F, U, s, W);
-    volume_targets(s, d);
-    float J[3][3], sq[3];
-    bool fr[3];
-    volume_jacobian(s, d, J, fr, sq);
-    // A = U^T dF W
-    float A[3][3], T1[3][3];
+    Hess H;
+    hess_terms(T, F, H);
+    hess_apply(H, T.ws + T.wv, dF, dP);
+    store_corners(dP, T, force + 4 * (int64_t)e);
+}
+
+// ---- preconditioned CG: one iteration in four launches beside the solve
+//
+// k_pcg_direction: beta = r.z / (r.z before), p = z + beta p, and the partial sums of m/dt^2 |p|^2
+// k_pcg_hvp:       per block of kLaTets tets (the plan of the local step) the per-vertex sums of d^2E[p]'s corner
+//                  forces, one per block-vertex entry, and the partial sums of (p at the vertex) . entry; p.Hp is the
+//                  two sums' total
+// k_pcg_update:    alpha = r.z / p.Hp, x += alpha p, r -= alpha (m/dt^2 p + the vertex's entries)
+// (the solve)      z = K^-1 r
+// k_dot_partial:   partial sums of r.z
+// Every block of the first and third adds the partial sums itself, in the same fixed order: no separate final
+// reduction, no Hp vector and no corner-force array.  p.Hp has to be that of the Hp that r gets (the energy
+// sum_e dF : dP differs from it by the rounding of the corner sums, and the last Newton corrections came out fifty
+// times noisier with it): it is taken from the stored entries, whose sum k_pcg_update rounds once.  The SVDs of a tet are taken once per solve (k_hvp_terms).
+// 50K-tet slab, one iteration: 80 us with thirteen launches (an SVD per tet in each; 9.5 + 9.1 us for H p and 14 us of
+// dots and vector updates, ncu), 48 us so; bound by the latency of nine dependent kernels.
+
+// (a fixed order: threads stride the array, then a tree)
+__device__ __forceinline__ double block_sum64(double v, double* sm /* 33 */) {
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    if (lane == 0) sm[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        v = lane < nw ? sm[lane] : 0.0;
 #pragma unroll
-        for (int j = 0; j < 3; ++j) T1[i][j] = dF[i][0] * W[0][j] + dF[i][1] * W[1][j] + dF[i][2] * W[2][j];
+        for (int o = 4; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);   // at most 8 warps
+        if (lane == 0) sm[32] = v;
+    }
+    __syncthreads();
+    const double t = sm[32];
+    __syncthreads();
+    return t;
+}
+
+__device__ __forceinline__ double partials_sum(const double* __restrict__ p, int n, const double* __restrict__ p2, int n2,
+                                               double* sm) {
+    double v = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) v += p[i];
+    for (int i = threadIdx.x; i < n2; i += blockDim.x) v += p2[i];
+    return block_sum64(v, sm);
+}
+
+__global__ void __launch_bounds__(128) k_hvp_terms(int n_t, const int4* __restrict__ tets,
+                                                   const float4* __restrict__ geo, const float4* __restrict__ x,
+                                                   float* __restrict__ hess) {
+    const int e = blockIdx.x * 128 + threadIdx.x;
+    if (e >= n_t) return;
+    const Tet T = load_tet(e, n_t, tets, geo);
+    float F[3][3];
+    tet_grad(T, x, F);
+    Hess H;
+    hess_terms(T, F, H);
+    float* h = hess + e;   // planes of n_t
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) A[i][j] = U[0][i] * T1[0][j] + U[1][i] * T1[1][j] + U[2][i] * T1[2][j];
-    // B = ws B_R + wv B_V (in the singular frame)
-    float B[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        float diag = 0.f;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) diag += J[i][k] * A[k][k];
-        B[i][i] = T.wv * diag;
+    for (int k = 0; k < 9; ++k) {
+        h[(int64_t)k * n_t] = H.U[k / 3][k % 3];
+        h[(int64_t)(9 + k) * n_t] = H.W[k / 3][k % 3];
     }
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int k = 0; k < 6; ++k) h[(int64_t)(18 + k) * n_t] = H.J[k];
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            if (i == j) continue;
-            const float sym = 0.5f * (A[i][j] + A[j][i]);
-            const float skw = 0.5f * (A[i][j] - A[j][i]);
-            float ssum = s[i] + s[j];
-            if (fabsf(ssum) < 1e-6f) ssum = copysignf(1e-6f, ssum);
-            const float betaR = 2.f / ssum;
-            const float betaV = (d[i] + d[j]) / ssum;
-            float alphaV;
-            if (fr[i] && fr[j] && sq[i] > 0.f && sq[j] > 0.f) {
-                // both on the + branch: (d_i - d_j)/(s_i - s_j) without cancellation
-                alphaV = 0.5f * (1.f + (s[i] + s[j]) / (sq[i] + sq[j]));
-            } else if (fabsf(s[i] - s[j]) > 1e-6f * fmaxf(1.f, fabsf(s[i]))) {
-                alphaV = (d[i] - d[j]) / (s[i] - s[j]);
-            } else {
-                alphaV = J[i][i] - J[i][j];
-            }
-            B[i][j] = T.ws * (betaR * skw) + T.wv * (alphaV * sym + betaV * skw);
+    for (int k = 0; k < 3; ++k) {
+        h[(int64_t)(24 + k) * n_t] = H.al[k];
+        h[(int64_t)(27 + k) * n_t] = H.be[k];
+    }
+}
+
+// sc[parity]: r.z of this iteration, sc[1 - parity]: of the one before
+__global__ void __launch_bounds__(256) k_pcg_direction(int n, const double* __restrict__ rz_part, int n_rz,
+                                                       double* __restrict__ sc, int parity, int first,
+                                                       const float* __restrict__ mh2, const float4* __restrict__ z,
+                                                       float4* __restrict__ p, double* __restrict__ mp_part) {
+    __shared__ double sm[33];
+    pdl_trigger();
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    const float m = i < n ? mh2[i] : 0.f;
+    pdl_wait();
+    float4 zi = make_float4(0.f, 0.f, 0.f, 0.f), pi = zi;
+    if (i < n) {               // (loads in flight during the reduction)
+        zi = z[i];
+        if (!first) pi = p[i];
+    }
+    const double rz = partials_sum(rz_part, n_rz, nullptr, 0, sm);
+    float be = 0.f;
+    if (!first) {
+        const double old = sc[1 - parity];
+        be = fabs(old) > 1e-300 ? (float)(rz / old) : 0.f;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) sc[parity] = rz;
+    double acc = 0.0;
+    if (i < n) {
+        const float4 q = make_float4(zi.x + be * pi.x, zi.y + be * pi.y, zi.z + be * pi.z, 0.f);
+        p[i] = q;
+        acc = (double)m * ((double)q.x * q.x + (double)q.y * q.y + (double)q.z * q.z);
+    }
+    acc = block_sum64(acc, sm);
+    if (threadIdx.x == 0) mp_part[blockIdx.x] = acc;
+}
+
+// s + e += a b with the rounding errors of both operations kept in e (Ogita, Rump, Oishi, "Accurate sum and dot
+// product", 2005): as exact as FP64 sums, without its slow pipe
+__device__ __forceinline__ void dot2_add(float a, float b, float& s, float& e) {
+    const float p = __fmul_rn(a, b), pe = __fmaf_rn(a, b, -p);
+    const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
+    e = __fadd_rn(e, __fadd_rn(pe, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z))));
+    s = t;
+}
+
+__global__ void __launch_bounds__(PDG_LA_TETS) k_pcg_hvp(int n_t, const int4* __restrict__ tets,
+                                                         const float4* __restrict__ geo, const float* __restrict__ hess,
+                                                         const float4* __restrict__ p, const int* __restrict__ vptr,
+                                                         const int* __restrict__ vert, const int* __restrict__ cptr,
+                                                         const uint16_t* __restrict__ corner, float4* __restrict__ part,
+                                                         double* __restrict__ php_part) {
+    constexpr int B = PDG_LA_TETS;
+    __shared__ float fx[4 * B], fy[4 * B], fz[4 * B];
+    __shared__ double sm[33];
+    pdl_trigger();
+    const int e = blockIdx.x * B + threadIdx.x, ec = min(e, n_t - 1);
+    const Tet T = load_tet(ec, n_t, tets, geo);
+    const float* h = hess + ec;
+    Hess H;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        H.U[k / 3][k % 3] = __ldg(h + (int64_t)k * n_t);
+        H.W[k / 3][k % 3] = __ldg(h + (int64_t)(9 + k) * n_t);
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) H.J[k] = __ldg(h + (int64_t)(18 + k) * n_t);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        H.al[k] = __ldg(h + (int64_t)(24 + k) * n_t);
+        H.be[k] = __ldg(h + (int64_t)(27 + k) * n_t);
+    }
+    const int j0 = __ldg(&vptr[blockIdx.x]), j1 = __ldg(&vptr[blockIdx.x + 1]);
+    pdl_wait();   // (the terms were written before the predecessor of this kernel's first launch ended)
+    float dF[3][3], dP[3][3];
+    tet_grad(T, p, dF);
+    hess_apply(H, T.ws + T.wv, dF, dP);
+    if (e < n_t) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            fx[4 * threadIdx.x + q] = dP[0][0] * T.g[q][0] + dP[0][1] * T.g[q][1] + dP[0][2] * T.g[q][2];
+            fy[4 * threadIdx.x + q] = dP[1][0] * T.g[q][0] + dP[1][1] * T.g[q][1] + dP[1][2] * T.g[q][2];
+            fz[4 * threadIdx.x + q] = dP[2][0] * T.g[q][0] + dP[2][1] * T.g[q][1] + dP[2][2] * T.g[q][2];
         }
-    // dP = (ws + wv) dF - U B W^T
-    float UB[3][3], dP[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) UB[i][j] = U[i][0] * B[0][j] + U[i][1] * B[1][j] + U[i][2] * B[2][j];
-    const float wsum = T.ws + T.wv;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-            dP[i][j] = wsum * dF[i][j] - (UB[i][0] * W[j][0] + UB[i][1] * W[j][1] + UB[i][2] * W[j][2]);
-    store_corners(dP, T, force + 4 * (int64_t)e);
+    }
+    __syncthreads();
+    float s = 0.f, c = 0.f;
+    for (int j = j0 + threadIdx.x; j < j1; j += B) {
+        const float4 pv = p[__ldg(&vert[j])];
+        float ax = 0.f, ay = 0.f, az = 0.f;
+        for (int k = __ldg(&cptr[j]); k < __ldg(&cptr[j + 1]); ++k) {
+            const int q = __ldg(&corner[k]);
+            ax += fx[q];
+            ay += fy[q];
+            az += fz[q];
+        }
+        part[j] = make_float4(ax, ay, az, 0.f);
+        dot2_add(pv.x, ax, s, c);
+        dot2_add(pv.y, ay, s, c);
+        dot2_add(pv.z, az, s, c);
+    }
+    const double tot = block_sum64((double)s + (double)c, sm);
+    if (threadIdx.x == 0) php_part[blockIdx.x] = tot;
+}
+
+__global__ void __launch_bounds__(256) k_pcg_update(int n, const double* __restrict__ sc, int parity,
+                                                    const double* __restrict__ mp_part, int n_mp,
+                                                    const double* __restrict__ php_part, int n_php,
+                                                    const float* __restrict__ mh2, const int* __restrict__ ent_ptr,
+                                                    const int* __restrict__ ent, const float4* __restrict__ part,
+                                                    const float4* __restrict__ p, float4* __restrict__ x,
+                                                    float4* __restrict__ r) {
+    __shared__ double sm[33];
+    pdl_trigger();
+    const int i = blockIdx.x * 256 + threadIdx.x, ic = min(i, n - 1);
+    const float m = mh2[ic];
+    const int k0 = ent_ptr[ic], k1 = ent_ptr[ic + 1];
+    pdl_wait();
+    const float4 pi = p[ic];   // (loads in flight during the reduction)
+    float4 xi = x[ic], ri = r[ic];
+    float hx = 0.f, hy = 0.f, hz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;
+    dot2_add(m, pi.x, hx, cx);
+    dot2_add(m, pi.y, hy, cy);
+    dot2_add(m, pi.z, hz, cz);
+    for (int k = k0; k < k1; ++k) {
+        const float4 f = part[ent[k]];
+        dot2_add(1.f, f.x, hx, cx);
+        dot2_add(1.f, f.y, hy, cy);
+        dot2_add(1.f, f.z, hz, cz);
+    }
+    hx += cx;
+    hy += cy;
+    hz += cz;
+    const double php = partials_sum(mp_part, n_mp, php_part, n_php, sm);
+    const float al = fabs(php) > 1e-300 ? (float)(sc[parity] / php) : 0.f;
+    if (i >= n) return;
+    xi.x += al * pi.x; xi.y += al * pi.y; xi.z += al * pi.z;
+    ri.x -= al * hx; ri.y -= al * hy; ri.z -= al * hz;
+    x[i] = xi;
+    r[i] = ri;
 }
 
 // out_i = sign * (mh2_i * (x_i - y_i) + sum_inc force), y_i = xprev_i + h vprev_i + h^2 g (free vertices)
@@ -253,6 +477,8 @@ constexpr int kDotBlocks = 512;
 __global__ void __launch_bounds__(256) k_dot_partial(int n, const float4* __restrict__ a, const float4* __restrict__ b,
                                                      double* __restrict__ partial) {
     __shared__ double sm[256];
+    pdl_trigger();
+    pdl_wait();
     double acc = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float4 u = a[i], v = b[i];
@@ -267,10 +493,9 @@ __global__ void __launch_bounds__(256) k_dot_partial(int n, const float4* __rest
     if (threadIdx.x == 0) partial[blockIdx.x] = sm[0];
 }
 
-// mode 0: sc[dst] = sum; mode 1: alpha = sc[0] / sum (sc[1] = sum, sc[2] = alpha);
-// mode 2: beta = sum / sc[0], sc[0] = sum (sc[3] = beta)
+// sc[dst] = sum of the partial sums
 __global__ void __launch_bounds__(256) k_dot_final(int nb, const double* __restrict__ partial, double* __restrict__ sc,
-                                                   int mode, int dst) {
+                                                   int dst) {
     __shared__ double sm[256];
     double acc = 0.0;
     for (int i = threadIdx.x; i < nb; i += blockDim.x) acc += partial[i];
@@ -280,41 +505,7 @@ __global__ void __launch_bounds__(256) k_dot_final(int nb, const double* __restr
         if (threadIdx.x < w) sm[threadIdx.x] += sm[threadIdx.x + w];
         __syncthreads();
     }
-    if (threadIdx.x != 0) return;
-    const double v = sm[0];
-    if (mode == 0) {
-        sc[dst] = v;
-    } else if (mode == 1) {
-        sc[1] = v;
-        sc[2] = (fabs(v) > 1e-300) ? sc[0] / v : 0.0;
-    } else {
-        sc[3] = (fabs(sc[0]) > 1e-300) ? v / sc[0] : 0.0;
-        sc[0] = v;
-    }
-}
-
-// x += alpha p ; r -= alpha Ap  (alpha = sc[2])
-__global__ void k_cg_update(int n, const double* __restrict__ sc, const float4* __restrict__ p,
-                            const float4* __restrict__ Ap, float4* __restrict__ x, float4* __restrict__ r) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float al = (float)sc[2];
-    const float4 pi = p[i], api = Ap[i];
-    float4 xi = x[i], ri = r[i];
-    xi.x += al * pi.x; xi.y += al * pi.y; xi.z += al * pi.z;
-    ri.x -= al * api.x; ri.y -= al * api.y; ri.z -= al * api.z;
-    x[i] = xi;
-    r[i] = ri;
-}
-
-// p = z + beta p (beta = sc[3]); beta_zero: p = z
-__global__ void k_cg_direction(int n, const double* __restrict__ sc, const float4* __restrict__ z,
-                               float4* __restrict__ p, int beta_zero) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float be = beta_zero ? 0.f : (float)sc[3];
-    const float4 zi = z[i], pi = p[i];
-    p[i] = make_float4(zi.x + be * pi.x, zi.y + be * pi.y, zi.z + be * pi.z, 0.f);
+    if (threadIdx.x == 0) sc[dst] = sm[0];
 }
 
 // rhs = dLdx + mh2 (2 lam1 - lam2)  (free vertices)
@@ -447,6 +638,8 @@ __global__ void __launch_bounds__(256) k_pdot_partial(int n, const float* __rest
                                                       const uint8_t* __restrict__ mask, int mode,
                                                       double* __restrict__ partial) {
     __shared__ double sm[256];
+    pdl_trigger();
+    pdl_wait();
     double acc = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         if (mask && !mask[i]) continue;
@@ -759,25 +952,38 @@ void launch_grad_gamma(const pd_mesh* m, const float* vol, const int* user_of_te
 
 int dot_blocks() { return kDotBlocks; }
 
-void launch_dot(int n, const float4* a, const float4* b, double* partial, double* sc, int mode, int dst,
-                cudaStream_t s) {
+// partial sums of a.b over the free vertices; returns their number
+int launch_dot_partial(int n, const float4* a, const float4* b, double* partial, cudaStream_t s) {
     const int blocks = std::max(1, std::min(kDotBlocks, nb(n, 256)));
-    k_dot_partial<<<blocks, 256, 0, s>>>(n, a, b, partial);
+    launch_pdl(k_dot_partial, dim3(blocks), dim3(256), 0, s, n, a, b, partial);
     PDG_CHECK_LAUNCH();
-    k_dot_final<<<1, 256, 0, s>>>(blocks, partial, sc, mode, dst);
+    return blocks;
+}
+
+void launch_dot(int n, const float4* a, const float4* b, double* partial, double* sc, int dst, cudaStream_t s) {
+    const int blocks = launch_dot_partial(n, a, b, partial, s);
+    k_dot_final<<<1, 256, 0, s>>>(blocks, partial, sc, dst);
     PDG_CHECK_LAUNCH();
 }
 
-void launch_cg_update(int n, const double* sc, const float4* p, const float4* Ap, float4* x, float4* r,
-                      cudaStream_t s) {
-    if (n <= 0) return;
-    k_cg_update<<<nb(n, 256), 256, 0, s>>>(n, sc, p, Ap, x, r);
+int hess_floats() { return kHessFloats; }
+int pcg_vertex_blocks(int n_free) { return std::max(1, nb(n_free, 256)); }
+
+void launch_hvp_terms(const pd_mesh* m, const float4* x, float* hess, cudaStream_t s) {
+    if (m->n_t <= 0) return;
+    k_hvp_terms<<<nb(m->n_t, 128), 128, 0, s>>>(m->n_t, m->d_tets.p, m->d_geo.p, x, hess);
     PDG_CHECK_LAUNCH();
 }
 
-void launch_cg_direction(int n, const double* sc, const float4* z, float4* p, int beta_zero, cudaStream_t s) {
-    if (n <= 0) return;
-    k_cg_direction<<<nb(n, 256), 256, 0, s>>>(n, sc, z, p, beta_zero);
+// The three launches of one iteration before the solve (see above): z, n_rz partial sums of r.z in, x and r advanced.
+void launch_pcg_step(const pd_mesh* m, pd_adjoint* a, int n_rz, int iteration, float4* x, cudaStream_t s) {
+    const int n = m->n_free, parity = iteration & 1, nv = pcg_vertex_blocks(n);
+    launch_pdl(k_pcg_direction, dim3(nv), dim3(256), 0, s, n, a->partial.p, n_rz, a->sc.p, parity, iteration == 0,
+               m->d_mh2.p, a->z.p, a->p.p, a->mp_part.p);
+    launch_pdl(k_pcg_hvp, dim3(m->la_blocks), dim3(PDG_LA_TETS), 0, s, m->n_t, m->d_tets.p, m->d_geo.p, a->hess.p,
+               a->p.p, m->d_la_vptr.p, m->d_la_vert.p, m->d_la_cptr.p, m->d_la_corner.p, a->ent_part.p, a->php_part.p);
+    launch_pdl(k_pcg_update, dim3(nv), dim3(256), 0, s, n, a->sc.p, parity, a->mp_part.p, nv, a->php_part.p,
+               m->la_blocks, m->d_mh2.p, a->ent_ptr.p, a->ent.p, a->ent_part.p, a->p.p, x, a->r.p);
     PDG_CHECK_LAUNCH();
 }
 

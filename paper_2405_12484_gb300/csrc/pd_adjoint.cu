@@ -20,11 +20,11 @@ void launch_hvp(const pd_mesh* m, const float4* x, const float4* v, float4* forc
 void launch_grad_gamma(const pd_mesh* m, const float* vol, const int* user_of_tet, const float4* x,
                        const float4* lam, float* gs, float* gv, cudaStream_t s);
 int dot_blocks();
-void launch_dot(int n, const float4* a, const float4* b, double* partial, double* sc, int mode, int dst,
-                cudaStream_t s);
-void launch_cg_update(int n, const double* sc, const float4* p, const float4* Ap, float4* x, float4* r,
-                      cudaStream_t s);
-void launch_cg_direction(int n, const double* sc, const float4* z, float4* p, int beta_zero, cudaStream_t s);
+int launch_dot_partial(int n, const float4* a, const float4* b, double* partial, cudaStream_t s);
+int hess_floats();
+int pcg_vertex_blocks(int n_free);
+void launch_hvp_terms(const pd_mesh* m, const float4* x, float* hess, cudaStream_t s);
+void launch_pcg_step(const pd_mesh* m, pd_adjoint* a, int n_rz, int iteration, float4* x, cudaStream_t s);
 void launch_adj_rhs(int n, const float4* dldx, const float* mh2, const float4* lam1, const float4* lam2, float4* rhs,
                     cudaStream_t s);
 void launch_grad_local64(const pd_mesh* m, const double* geo64, const double* x64, double* force64, cudaStream_t s);
@@ -61,16 +61,11 @@ void adjoint_pcg(pd_mesh* m, pd_adjoint* a, const float4* x_lin, const float4* b
     PDG_CUDA(cudaMemsetAsync(x, 0, sizeof(float4) * m->n_v, s));
     if (n <= 0) return;
     PDG_CUDA(cudaMemcpyAsync(a->r.p, b, sizeof(float4) * n, cudaMemcpyDeviceToDevice, s));
-    launch_dd_solve(m, a->r.p, a->z.p, s, false);
-    launch_cg_direction(n, a->sc.p, a->z.p, a->p.p, 1, s);
-    launch_dot(n, a->r.p, a->z.p, a->partial.p, a->sc.p, 0, 0, s);
+    launch_hvp_terms(m, x_lin, a->hess.p, s);
     for (int k = 0; k < a->cg_iters; ++k) {
-        launch_hvp(m, x_lin, a->p.p, m->d_force.p, a->Ap.p, s);
-        launch_dot(n, a->p.p, a->Ap.p, a->partial.p, a->sc.p, 1, 0, s);
-        launch_cg_update(n, a->sc.p, a->p.p, a->Ap.p, x, a->r.p, s);
         launch_dd_solve(m, a->r.p, a->z.p, s, false);
-        launch_dot(n, a->r.p, a->z.p, a->partial.p, a->sc.p, 2, 0, s);
-        launch_cg_direction(n, a->sc.p, a->z.p, a->p.p, 0, s);
+        const int n_rz = launch_dot_partial(n, a->r.p, a->z.p, a->partial.p, s);
+        launch_pcg_step(m, a, n_rz, k, x, s);
     }
 }
 
@@ -149,7 +144,7 @@ pd_status pd_adjoint_create(pd_mesh* m, int32_t cg_iters, pd_adjoint** out) {
         a->cg_iters = cg_iters;
         const size_t nv = (size_t)m->n_v;
         DBuf<float4>* bufs[] = {&a->xeq, &a->vprev, &a->g, &a->rhs, &a->lam, &a->lam1, &a->lam2,
-                                &a->r, &a->z, &a->p, &a->Ap, &a->dx};
+                                &a->r, &a->z, &a->p, &a->dx};
         for (auto* b : bufs) {
             b->alloc(nv);
             PDG_CUDA(cudaMemsetAsync(b->p, 0, sizeof(float4) * nv, m->stream));
@@ -157,6 +152,22 @@ pd_status pd_adjoint_create(pd_mesh* m, int32_t cg_iters, pd_adjoint** out) {
         a->partial.alloc(dot_blocks());
         a->sc.alloc(8);
         PDG_CUDA(cudaMemsetAsync(a->sc.p, 0, sizeof(double) * 8, m->stream));
+        a->hess.alloc((size_t)hess_floats() * m->n_t);
+        a->ent_part.alloc(m->la_entries);
+        a->mp_part.alloc(pcg_vertex_blocks(m->n_free));
+        a->php_part.alloc(std::max(m->la_blocks, 1));
+        // the local plan's block-vertex entries by vertex, in block order
+        std::vector<int32_t> vert(m->la_entries), eptr(m->n_free + 1, 0), ent(m->la_entries);
+        if (m->la_entries > 0)
+            PDG_CUDA(cudaMemcpyAsync(vert.data(), m->d_la_vert.p, sizeof(int32_t) * m->la_entries,
+                                     cudaMemcpyDeviceToHost, m->stream));
+        PDG_CUDA(cudaStreamSynchronize(m->stream));
+        for (int32_t v : vert) ++eptr[v + 1];
+        for (int32_t i = 0; i < m->n_free; ++i) eptr[i + 1] += eptr[i];
+        std::vector<int32_t> fill(eptr.begin(), eptr.end() - 1);
+        for (int32_t j = 0; j < m->la_entries; ++j) ent[fill[vert[j]]++] = j;
+        upload(a->ent_ptr, eptr, m->stream);
+        upload(a->ent, ent, m->stream);
         std::vector<float> vol(m->n_t);
         for (int32_t t = 0; t < m->n_t; ++t) vol[t] = (float)m->vol[t];
         a->vol.alloc(m->n_t);

@@ -16,8 +16,7 @@
 namespace pdg {
 
 int dot_blocks();
-void launch_dot(int n, const float4* a, const float4* b, double* partial, double* sc, int mode, int dst,
-                cudaStream_t s);
+void launch_dot(int n, const float4* a, const float4* b, double* partial, double* sc, int dst, cudaStream_t s);
 int gn_scalar_count();
 int gn_partial_blocks();
 void launch_gn_setup(const pd_mesh* m, const float* vol, const float4* x, float* Ts, float* Tv, cudaStream_t s);
@@ -92,10 +91,10 @@ static void gn_apply(pd_mesh* m, pd_adjoint* a, const float* v, const uint8_t* a
     const int nf = m->n_free;
     double* sc = a->gn_sc.p;
     launch_gn_bv(m, a->gn_Ts.p, a->gn_Tv.p, a->user_of_tet.p, v, m->d_force.p, a->gn_b.p, s);
-    launch_dot(nf, a->gn_b.p, a->gn_b.p, a->gn_partial.p, sc, 0, S_N1, s);
+    launch_dot(nf, a->gn_b.p, a->gn_b.p, a->gn_partial.p, sc, S_N1, s);
     launch_normalize_f4(nf, sc, S_N1, a->gn_b.p, s);
     adjoint_pcg(m, a, a->xeq.p, a->gn_b.p, a->gn_mu.p, s);      // mu / |B v|
-    launch_dot(nf, a->gn_mu.p, a->gn_mu.p, a->gn_partial.p, sc, 0, S_N2, s);
+    launch_dot(nf, a->gn_mu.p, a->gn_mu.p, a->gn_partial.p, sc, S_N2, s);
     launch_normalize_f4(nf, sc, S_N2, a->gn_mu.p, s);
     adjoint_pcg(m, a, a->xeq.p, a->gn_mu.p, a->gn_nu.p, s);     // nu / (g_scale |B v| |mu|)
     launch_gn_btv(m, a->gn_Ts.p, a->gn_Tv.p, a->user_of_tet.p, a->gn_nu.p, active, sc, S_N1, S_N2, g_scale, out, s);

@@ -567,7 +567,13 @@ struct pd_mesh {
 struct pd_adjoint {
     pd_mesh* mesh = nullptr;
     int32_t cg_iters = 30;
-    pdg::DBuf<float4> xeq, vprev, g, rhs, lam, lam1, lam2, r, z, p, Ap, dx;
+    pdg::DBuf<float4> xeq, vprev, g, rhs, lam, lam1, lam2, r, z, p, dx;
+    // one CG iteration: per-tet Hessian terms, the sums of the local plan's block-vertex entries and the entries of
+    // every free vertex, partial sums of the scalars
+    pdg::DBuf<float> hess;
+    pdg::DBuf<float4> ent_part;
+    pdg::DBuf<int32_t> ent_ptr, ent;
+    pdg::DBuf<double> mp_part, php_part;
     pdg::DBuf<double> partial, sc;
     pdg::DBuf<float> vol;
     pdg::DBuf<int32_t> user_of_tet;
