@@ -40,7 +40,7 @@ constexpr int kProjThreads = 128;
 
 __global__ void __launch_bounds__(kProjThreads) k_project(const float* __restrict__ Fin, int n, float* __restrict__ Rout,
                                                           float* __restrict__ Vout, float* __restrict__ sout) {
-    __shared__ float buf[9 * kProjThreads];
+    __shared__ float buf[21 * kProjThreads];
     const int64_t e0 = (int64_t)blockIdx.x * kProjThreads;
     const int ne = (int)min((int64_t)kProjThreads, n - e0), tid = threadIdx.x;
     for (int l = tid; l < 9 * ne; l += kProjThreads) buf[l] = Fin[9 * e0 + l];
@@ -66,27 +66,23 @@ __global__ void __launch_bounds__(kProjThreads) k_project(const float* __restric
         volume_targets(s, d);
         udwt(U, d, W, V);
     }
-    if (Rout) {
-        __syncthreads();
+    // all three results in their own parts of the buffer: one exchange
+    float *bR = buf, *bV = buf + 9 * kProjThreads, *bs = buf + 18 * kProjThreads;
+    __syncthreads();           // the inputs have been read
 #pragma unroll
-        for (int i = 0; i < 9; ++i) buf[9 * tid + i] = R[i / 3][i % 3];
-        __syncthreads();
-        for (int l = tid; l < 9 * ne; l += kProjThreads) Rout[9 * e0 + l] = buf[l];
+    for (int i = 0; i < 9; ++i) {
+        bR[9 * tid + i] = R[i / 3][i % 3];
+        bV[9 * tid + i] = V[i / 3][i % 3];
     }
-    if (Vout) {
-        __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 9; ++i) buf[9 * tid + i] = V[i / 3][i % 3];
-        __syncthreads();
-        for (int l = tid; l < 9 * ne; l += kProjThreads) Vout[9 * e0 + l] = buf[l];
-    }
-    if (sout) {
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 3; ++i) buf[3 * tid + i] = s[i];
-        __syncthreads();
-        for (int l = tid; l < 3 * ne; l += kProjThreads) sout[3 * e0 + l] = buf[l];
-    }
+    for (int i = 0; i < 3; ++i) bs[3 * tid + i] = s[i];
+    __syncthreads();
+    if (Rout)
+        for (int l = tid; l < 9 * ne; l += kProjThreads) Rout[9 * e0 + l] = bR[l];
+    if (Vout)
+        for (int l = tid; l < 9 * ne; l += kProjThreads) Vout[9 * e0 + l] = bV[l];
+    if (sout)
+        for (int l = tid; l < 3 * ne; l += kProjThreads) sout[3 * e0 + l] = bs[l];
 }
 
 // geo holds three float4 rows per tet in SoA blocks:
