@@ -45,25 +45,6 @@ __global__ void k_inertia(int n_v, int n_free, float h, float gx, float gy, floa
     }
 }
 
-// by0 = (m/h^2) y - K_fp x_p for a given y (diagnostic path); pinned x_p from x.
-__global__ void k_by0(int n_free, const float4* __restrict__ y, const float4* __restrict__ xpin,
-                      const float* __restrict__ mh2, const int* __restrict__ kfp_ptr, const int* __restrict__ kfp_col,
-                      const float* __restrict__ kfp_val, float4* __restrict__ by0) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_free) return;
-    float4 yy = y[i];
-    float m = mh2[i];
-    float4 acc = f4(m * yy.x, m * yy.y, m * yy.z);
-    for (int k = kfp_ptr[i]; k < kfp_ptr[i + 1]; ++k) {
-        float kv = kfp_val[k];
-        float4 p = xpin[kfp_col[k]];
-        acc.x -= kv * p.x;
-        acc.y -= kv * p.y;
-        acc.z -= kv * p.z;
-    }
-    by0[i] = acc;
-}
-
 __global__ void k_velocity(int n_v, float inv_h, const float4* __restrict__ x, const float4* __restrict__ xprev,
                            float4* __restrict__ v, int* __restrict__ err) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -109,6 +90,60 @@ __global__ void k_gather_in(int n_v, const int* __restrict__ old_of_new, const f
     dst[i] = f4(src[3 * (int64_t)o], src[3 * (int64_t)o + 1], src[3 * (int64_t)o + 2]);
 }
 
+// Two vertex arrays at once (either may be null): the state in and out in one launch each (a launch of 98K vertices
+// takes 3.3 us, nearly all of it latency).
+__global__ void k_gather_in2(int n_v, const int* __restrict__ old_of_new, const float* __restrict__ a,
+                             const float* __restrict__ b, float4* __restrict__ da, float4* __restrict__ db) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n_v) return;
+    const int64_t o = 3 * (int64_t)old_of_new[i];
+    if (a) da[i] = f4(a[o], a[o + 1], a[o + 2]);
+    if (b) db[i] = f4(b[o], b[o + 1], b[o + 2]);
+}
+
+__global__ void k_scatter_out2(int n_v, const int* __restrict__ old_of_new, const float4* __restrict__ a,
+                               const float4* __restrict__ b, float* __restrict__ da, float* __restrict__ db) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n_v) return;
+    const int64_t o = 3 * (int64_t)old_of_new[i];
+    if (da) {
+        const float4 u = a[i];
+        da[o] = u.x;
+        da[o + 1] = u.y;
+        da[o + 2] = u.z;
+    }
+    if (db) {
+        const float4 u = b[i];
+        db[o] = u.x;
+        db[o + 1] = u.y;
+        db[o + 2] = u.z;
+    }
+}
+
+// Inputs of the local step alone, from the caller's arrays: positions x in library order, and
+// by0 = (m/h^2) y - K_fp x_p with the pinned positions of x.  One launch for two gathers, the copy of the pinned
+// positions and the product (pd_local_rhs of the 390K shell: 63 us a call with four, 54 us so).
+__global__ void k_local_inputs(int n_v, int n_free, const int* __restrict__ old_of_new, const float* __restrict__ x,
+                               const float* __restrict__ y, const float* __restrict__ mh2,
+                               const int* __restrict__ kfp_ptr, const int* __restrict__ kfp_col,
+                               const float* __restrict__ kfp_val, float4* __restrict__ xi, float4* __restrict__ by0) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n_v) return;
+    const int64_t o = 3 * (int64_t)old_of_new[i];
+    xi[i] = f4(x[o], x[o + 1], x[o + 2]);
+    if (i >= n_free) return;
+    const float m = mh2[i];
+    float4 acc = f4(m * y[o], m * y[o + 1], m * y[o + 2]);
+    for (int k = kfp_ptr[i]; k < kfp_ptr[i + 1]; ++k) {
+        const float kv = kfp_val[k];
+        const int64_t q = 3 * (int64_t)old_of_new[n_free + kfp_col[k]];
+        acc.x -= kv * x[q];
+        acc.y -= kv * x[q + 1];
+        acc.z -= kv * x[q + 2];
+    }
+    by0[i] = acc;
+}
+
 // geo[t].w = V_e gamma_s, geo[n_t + t].w = V_e gamma_v (inputs already in sorted tet order)
 __global__ void k_weights(int n_t, const float* __restrict__ vol, const float* __restrict__ gs,
                           const float* __restrict__ gv, float4* __restrict__ geo) {
@@ -129,11 +164,19 @@ void launch_inertia(const pd_mesh* m, float h, float gx, float gy, float gz, cud
     PDG_CHECK_LAUNCH();
 }
 
-void launch_by0_from_y(const pd_mesh* m, const float4* y, float4* by0, cudaStream_t s) {
-    if (m->n_free <= 0) return;
-    // pinned positions come from the pin-target buffer (filled by the caller)
-    k_by0<<<nblk(m->n_free, 256), 256, 0, s>>>(m->n_free, y, m->d_pin_tgt.p, m->d_mh2.p, m->d_kfp_ptr.p,
-                                               m->d_kfp_col.p, m->d_kfp_val.p, by0);
+void launch_local_inputs(const pd_mesh* m, const float* x, const float* y, float4* xi, float4* by0, cudaStream_t s) {
+    k_local_inputs<<<nblk(m->n_v, 256), 256, 0, s>>>(m->n_v, m->n_free, m->d_old_of_new.p, x, y, m->d_mh2.p,
+                                                     m->d_kfp_ptr.p, m->d_kfp_col.p, m->d_kfp_val.p, xi, by0);
+    PDG_CHECK_LAUNCH();
+}
+
+void launch_state_in(const pd_mesh* m, const float* x, const float* v, cudaStream_t s) {
+    k_gather_in2<<<nblk(m->n_v, 256), 256, 0, s>>>(m->n_v, m->d_old_of_new.p, x, v, m->d_x.p, m->d_v.p);
+    PDG_CHECK_LAUNCH();
+}
+
+void launch_state_out(const pd_mesh* m, float* x, float* v, cudaStream_t s) {
+    k_scatter_out2<<<nblk(m->n_v, 256), 256, 0, s>>>(m->n_v, m->d_old_of_new.p, m->d_x.p, m->d_v.p, x, v);
     PDG_CHECK_LAUNCH();
 }
 

@@ -517,6 +517,8 @@ struct pd_mesh {
     // vectors of pd_local_rhs and pd_solve (n_v each; both calls end with a synchronisation), allocated on first use
     // and kept: two or five cudaMalloc / cudaFree pairs took 0.3 ms of a 0.4 ms solve, 0.45 of a 0.5 ms local step
     pdg::DBuf<float4> d_io[4];
+    cudaGraphExec_t solve_graph = nullptr;   // the solve between them (see pd_solve); dropped by pd_prefactor
+    int32_t solve_calls = 0;                 // calls of pd_solve since pd_prefactor
 
     // generations of the FP32 state (pd_set_state, pd_step) and of the
     // materials (pd_set_materials): the adjoint workspace's FP64 state and
@@ -620,7 +622,9 @@ void launch_pin_copy(const pd_mesh* m, const float* user_targets, cudaStream_t s
 void launch_pin_hold(const pd_mesh* m, cudaStream_t s);
 void launch_scatter_out(const pd_mesh* m, const float4* src, float* dst, int free_only, cudaStream_t s);
 void launch_gather_in(const pd_mesh* m, const float* src, float4* dst, cudaStream_t s);
-void launch_by0_from_y(const pd_mesh* m, const float4* y, float4* by0, cudaStream_t s);
+void launch_local_inputs(const pd_mesh* m, const float* x, const float* y, float4* xi, float4* by0, cudaStream_t s);
+void launch_state_in(const pd_mesh* m, const float* x, const float* v, cudaStream_t s);
+void launch_state_out(const pd_mesh* m, float* x, float* v, cudaStream_t s);
 
 // subspace solve: b (free, new order) -> x positions of free vertices written into `xout`
 // (float4 array indexed by new vertex id).
