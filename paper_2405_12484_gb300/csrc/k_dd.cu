@@ -388,8 +388,8 @@ static_assert(kAxM == 1, "the tiled layout has one output chunk per block");
 
 // ring bytes of a launch whose widest tile has wmax outputs (a multiple of VN)
 template <class T>
-inline size_t axt_ring_bytes(int wmax) {
-    const size_t ring = (size_t)kAxtStages * kAxtRows * wmax * sizeof(T);
+inline size_t axt_ring_bytes(int wmax, int stage_rows) {
+    const size_t ring = (size_t)kAxtStages * stage_rows * wmax * sizeof(T);
     const size_t red = (size_t)(kAxtWarps - 1) * wmax * 3 * sizeof(float);
     return (std::max(ring, red) + 15) / 16 * 16;
 }
@@ -399,10 +399,10 @@ __global__ void __launch_bounds__(32 * (kAxtWarps + 1)) k_axpy_tma(const AxDesc*
                                                                    const AxBlock* __restrict__ blocks,
                                                                    AxBases single,
                                                                    const AxBases* __restrict__ multi,
-                                                                   int ring_bytes, int* __restrict__ err) {
+                                                                   int ring_bytes, int R, int* __restrict__ err) {
     using namespace tma;
     constexpr int VN = VecN<T>::N;
-    constexpr int S = kAxtStages, R = kAxtRows;
+    constexpr int S = kAxtStages;
     extern __shared__ __align__(128) unsigned char axt_smem[];
     T* ring = reinterpret_cast<T*>(axt_smem);
     float* red = reinterpret_cast<float*>(axt_smem);     // reused after the last stage
@@ -569,10 +569,18 @@ constexpr int kAxfRows = kAxtRows;
 // lanes whose A operand is not zero: groups 0..2 (x, y, z in rows g and g + 8)
 constexpr int kAxmFragLanes = 12;
 
-inline size_t axm_ring_bytes(int wmax, bool tf32 = false) {
-    const size_t b = tf32 ? (size_t)kAxmStages * kAxfRows * wmax * sizeof(float)
-                          : (size_t)kAxmStages * kAxmRows * wmax * sizeof(__nv_bfloat16);
+inline size_t axm_ring_bytes(int wmax, bool tf32, int stage_rows) {
+    const size_t b = (size_t)kAxmStages * stage_rows * wmax * (tf32 ? sizeof(float) : sizeof(__nv_bfloat16));
     return (b + 15) / 16 * 16;
+}
+
+// Rows per stage of a launch (a multiple of `unit`; the results do not depend on it).  With many blocks per SM the
+// short stages of `unit` rows keep enough copies in flight; with less than two, a block alone waits for the latency of
+// each round of three stages (a 455-row tile in fifteen stages of 32 rows), so the stages grow to 64 KB a ring.
+inline int ax_stage_rows(int n_blocks, int sms, int k_max, int w_max, int elem, int unit) {
+    if (n_blocks >= 2 * sms) return unit;
+    const int fit = 65536 / (kAxtStages * std::max(w_max, 1) * elem) / unit * unit;
+    return std::max(unit, std::min(fit, (k_max + unit - 1) / unit * unit));
 }
 
 __device__ __forceinline__ uint32_t to_tf32(float x) {
@@ -597,12 +605,12 @@ __device__ __forceinline__ void mma_tf32_1688(float (&d)[4], const uint4& a, uin
 template <bool TF32>
 __global__ void __launch_bounds__(32 * (kAxtWarps + 1)) k_axpy_mma(const AxDesc* __restrict__ descs,
                                                                    const AxBlock* __restrict__ blocks, AxBases B,
-                                                                   int ring_bytes, int* __restrict__ err) {
+                                                                   int ring_bytes, int R, int* __restrict__ err) {
     using namespace tma;
     using E = typename std::conditional<TF32, float, __nv_bfloat16>::type;
     constexpr int KB = TF32 ? 8 : 16;   // matrix rows per mma k-block
-    constexpr int S = kAxmStages, R = TF32 ? kAxfRows : kAxmRows;
-    static_assert(R % KB == 0, "stages hold whole k-blocks");
+    constexpr int S = kAxmStages;
+    static_assert((TF32 ? kAxfRows : kAxmRows) % KB == 0, "stages hold whole k-blocks (R is a multiple of these rows)");
     extern __shared__ __align__(128) unsigned char axm_smem[];
     __shared__ __align__(8) uint64_t full[S], empty[S];
     __shared__ int abort_flag;
@@ -1536,7 +1544,7 @@ int axm_smem_limit() {
 
 template <class T>
 void launch_ax(const AxDesc* descs, const AxBlock* blocks, int n_blocks, int k_max, const AxBases& B, cudaStream_t s,
-               int* tma_err = nullptr, int w_max = 0, bool pdl = false, bool tf32 = false) {
+               int* tma_err = nullptr, int w_max = 0, bool pdl = false, bool tf32 = false, int sms = 0) {
     if (n_blocks <= 0) return;
     const bool bf16 = std::is_same<T, __nv_bfloat16>::value;
     if (tma_err && (bf16 || tf32)) {
@@ -1544,25 +1552,27 @@ void launch_ax(const AxDesc* descs, const AxBlock* blocks, int n_blocks, int k_m
         // the A operands take 16 bytes per k-block for each of lanes 0..11)
         const int kb = bf16 ? 16 : 8;
         const int kp = (std::max(k_max, 1) + kb - 1) / kb * kb;
-        const size_t ring = axm_ring_bytes(w_max, !bf16);
+        const int rows = ax_stage_rows(n_blocks, sms, kp, w_max, bf16 ? 2 : 4, bf16 ? kAxmRows : kAxfRows);
+        const size_t ring = axm_ring_bytes(w_max, !bf16, rows);
         const size_t smem = ring + (size_t)(kp / kb) * kAxmFragLanes * sizeof(uint4) + sizeof(float4) * std::max(k_max, 1);
         if ((int)smem > axm_smem_limit()) throw Fail{PD_ERR_UNSUPPORTED};
         auto kern = bf16 ? k_axpy_mma<false> : k_axpy_mma<true>;
         if (pdl)
-            launch_pdl(kern, dim3(n_blocks), dim3(32 * (kAxtWarps + 1)), smem, s, descs, blocks, B, (int)ring,
+            launch_pdl(kern, dim3(n_blocks), dim3(32 * (kAxtWarps + 1)), smem, s, descs, blocks, B, (int)ring, rows,
                        tma_err);
         else
-            kern<<<n_blocks, 32 * (kAxtWarps + 1), smem, s>>>(descs, blocks, B, (int)ring, tma_err);
+            kern<<<n_blocks, 32 * (kAxtWarps + 1), smem, s>>>(descs, blocks, B, (int)ring, rows, tma_err);
     } else if (tma_err) {
         // tiled matrices: the bulk-copy streaming kernel
-        const size_t ring = axt_ring_bytes<T>(w_max);
+        const int rows = ax_stage_rows(n_blocks, sms, k_max, w_max, sizeof(T), kAxtRows);
+        const size_t ring = axt_ring_bytes<T>(w_max, rows);
         const size_t smem = ring + sizeof(float4) * std::max(k_max, 1);
         if ((int)smem > axt_smem_limit<T>()) throw Fail{PD_ERR_UNSUPPORTED};
         if (pdl)
             launch_pdl(k_axpy_tma<T, false>, dim3(n_blocks), dim3(32 * (kAxtWarps + 1)), smem, s, descs, blocks, B,
-                       (const AxBases*)nullptr, (int)ring, tma_err);
+                       (const AxBases*)nullptr, (int)ring, rows, tma_err);
         else
-            k_axpy_tma<T, false><<<n_blocks, 32 * (kAxtWarps + 1), smem, s>>>(descs, blocks, B, nullptr, (int)ring,
+            k_axpy_tma<T, false><<<n_blocks, 32 * (kAxtWarps + 1), smem, s>>>(descs, blocks, B, nullptr, (int)ring, rows,
                                                                               tma_err);
     } else {
         k_axpy_form<T, false><<<n_blocks, 32 * kAxWarps, sizeof(float4) * std::max(k_max, 1), s>>>(descs, blocks, B,
@@ -1680,7 +1690,7 @@ void dd_solve_impl(pd_mesh* m, const T* pool, const float4* b, float4* xout, con
                 phase_begin(m, PH_INTERIOR, m->side[0]);   // (timed per launch)
                 launch_ax<T>(m->d_ax_desc_int.p, m->d_ax_blk_int.p + b0, std::min(per, nb - b0), m->ax_kmax_int,
                              product(pool, b, nullptr, nullptr, w.tc, true, false), m->side[0], m->ax_tiled ? m->d_err.p : nullptr,
-                             m->ax_wmax_int, false, m->ax_tf32);
+                             m->ax_wmax_int, false, m->ax_tf32, m->sms);
                 phase_end(m, m->side[0]);
             }
         }
@@ -1690,7 +1700,7 @@ void dd_solve_impl(pd_mesh* m, const T* pool, const float4* b, float4* xout, con
         phase_begin(m, PH_CONDENSE, s);
         launch_ax<T>(m->d_ax_desc_cond.p, m->d_ax_blk_cond.p, m->ax_blocks_cond, m->ax_kmax_cond,
                      product(pool, b, nullptr, nullptr, w.tc, true, direct), s, m->ax_tiled ? m->d_err.p : nullptr, m->ax_wmax_cond,
-                     true, m->ax_tf32);
+                     true, m->ax_tf32, m->sms);
         phase_end(m, s);
     }
     if (m->n_B > 0) {
@@ -1752,7 +1762,7 @@ void dd_solve_impl(pd_mesh* m, const T* pool, const float4* b, float4* xout, con
         phase_begin(m, PH_BACKSUB, s);
         launch_ax<T>(m->d_ax_desc_back.p, m->d_ax_blk_back.p, m->ax_blocks_back, m->ax_kmax_back,
                      product(pool, xout + m->n_int, m->d_bidx.p, w.tc, xout, true, false), s, m->ax_tiled ? m->d_err.p : nullptr,
-                     m->ax_wmax_back, true, m->ax_tf32);
+                     m->ax_wmax_back, true, m->ax_tf32, m->sms);
         phase_end(m, s);
     }
     const int S = (int)m->jacobi_omega.size();
@@ -1793,13 +1803,13 @@ void launch_dd_solve_scratch(pd_mesh* m, const float4* b, float4* xout, float4* 
 void launch_axpy_b(const AxDesc* descs, const AxBlock* blocks, const AxBases* bases, int n_blocks, int k_max,
                    int w_max, int* err, bool late, cudaStream_t s) {
     if (n_blocks <= 0) return;
-    const size_t ring = axt_ring_bytes<float>(w_max);
+    const size_t ring = axt_ring_bytes<float>(w_max, kAxtRows);
     const size_t smem = ring + sizeof(float4) * std::max(k_max, 1);
     if ((int)smem > axt_smem_limit<float>()) throw Fail{PD_ERR_UNSUPPORTED};
     AxBases launch{};
     launch.late = late;
     launch_pdl(k_axpy_tma<float, true>, dim3(n_blocks), dim3(32 * (kAxtWarps + 1)), smem, s, descs, blocks, launch, bases,
-               (int)ring, err);
+               (int)ring, kAxtRows, err);
     PDG_CHECK_LAUNCH();
 }
 

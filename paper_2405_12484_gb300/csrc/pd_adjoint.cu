@@ -62,11 +62,44 @@ void adjoint_pcg(pd_mesh* m, pd_adjoint* a, const float4* x_lin, const float4* b
     if (n <= 0) return;
     PDG_CUDA(cudaMemcpyAsync(a->r.p, b, sizeof(float4) * n, cudaMemcpyDeviceToDevice, s));
     launch_hvp_terms(m, x_lin, a->hess.p, s);
-    for (int k = 0; k < a->cg_iters; ++k) {
-        launch_dd_solve(m, a->r.p, a->z.p, s, false);
-        const int n_rz = launch_dot_partial(n, a->r.p, a->z.p, a->partial.p, s);
-        launch_pcg_step(m, a, n_rz, k, x, s);
+    auto iteration = [&](int k, cudaStream_t q) {
+        launch_dd_solve(m, a->r.p, a->z.p, q, false);
+        const int n_rz = launch_dot_partial(n, a->r.p, a->z.p, a->partial.p, q);
+        launch_pcg_step(m, a, n_rz, k, x, q);
+    };
+    iteration(0, s);
+    // From the third solve for this vector after a prefactorisation on, pairs of iterations (an odd and an even one)
+    // are replayed as a graph, which takes thirteen launches and four event calls an iteration from the host
+    // (equilibrium and adjoint step of the 50K-tet slab: 8.1 ms with plain launches, 7.9 so).
+    constexpr int kPlainSolves = 2;
+    int k = 1;
+    if (m->use_graphs && a->cg_iters >= 3) {
+        if (a->pcg_gen != m->factor_gen) {
+            a->drop_pcg_graphs();
+            a->pcg_gen = m->factor_gen;
+        }
+        pd_adjoint::PcgGraph& G = a->pcg_graphs[x];
+        if (!G.exec && ++G.solves > kPlainSolves) {
+            cudaGraph_t graph = nullptr;
+            PDG_CUDA(cudaStreamBeginCapture(m->cap_stream, cudaStreamCaptureModeThreadLocal));
+            try {
+                iteration(1, m->cap_stream);
+                iteration(2, m->cap_stream);
+            } catch (...) {
+                cudaStreamEndCapture(m->cap_stream, &graph);
+                if (graph) cudaGraphDestroy(graph);
+                throw;
+            }
+            PDG_CUDA(cudaStreamEndCapture(m->cap_stream, &graph));
+            const cudaError_t e =
+                cudaGraphInstantiate(&G.exec, graph, m->node_priority ? cudaGraphInstantiateFlagUseNodePriority : 0);
+            cudaGraphDestroy(graph);
+            PDG_CUDA(e);
+        }
+        if (G.exec)
+            for (; k + 1 < a->cg_iters; k += 2) PDG_CUDA(cudaGraphLaunch(G.exec, s));
     }
+    for (; k < a->cg_iters; ++k) iteration(k, s);
 }
 
 // FP64 side of the workspace: buffers on first use, per-tet operators after

@@ -752,6 +752,7 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
     if (m->solve_graph) cudaGraphExecDestroy(m->solve_graph);
     m->solve_graph = nullptr;
     m->solve_calls = 0;
+    ++m->factor_gen;
     const int32_t n_free = m->n_free, n_int = m->n_int, n_B = m->n_B, n_dom = m->n_dom;
     const double inv_h2 = 1.0 / (dt * dt);
 
@@ -1063,15 +1064,33 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
     m->ax_tiled = tiled;
     m->ax_tf32 = fragT;
     if (tiled) ax_prepare_tma(m->prec);
-    auto cast_ax = [&](const double* src, int lds, int rows, int cols, int transpose, int64_t off, int ld) {
+    // Outputs per tile of the boundary-mode and back-substitution products: the widest (OWt) that still gives a launch
+    // a block per SM, down to 32 (a block streams its tile alone, so few and wide tiles leave most SMs idle).  Not the
+    // interior product, which runs beside the chain, nor a serving request, whose tiles share a launch with others' (six
+    // requests 42 ms with wide tiles, 49 with narrow ones).  The results do not depend on it.  20 iterations with
+    // 128-output tiles and stages of 32 rows / so, with the longer stages of ax_stage_rows: 53K-tet shell FP32 556 /
+    // 513 us, TF32 607 / 554, 27K slab 498 / 451, 10 of the small slab 182 / 169.
+    auto tile_outputs = [&](auto&& outputs) {
+        int ow = OWt;
+        for (; ow > 32 && !m->batched_only; ow /= 2) {
+            int64_t blocks = 0;
+            for (int32_t d = 0; d < n_dom; ++d)
+                if (m->dom_n_int[d] > 0) blocks += (outputs(d) + ow - 1) / ow;
+            if (blocks >= m->sms) break;
+        }
+        return ow;
+    };
+    const int OWc = tile_outputs([&](int32_t d) { return (int)m->dom_bnd[d].size(); });
+    const int OWb = tile_outputs([&](int32_t d) { return (int)m->dom_n_int[d]; });
+    auto cast_ax = [&](const double* src, int lds, int rows, int cols, int transpose, int64_t off, int ld, int ow) {
         if (frag16)
-            launch_cast_frag16(src, lds, rows, cols, transpose, m->d_mat16.p, off, ax_chunk_width(cols, OWt, VNt),
+            launch_cast_frag16(src, lds, rows, cols, transpose, m->d_mat16.p, off, ax_chunk_width(cols, ow, VNt),
                                s);
         else if (fragT)
-            launch_cast_frag32(src, lds, rows, cols, transpose, m->d_mat32.p, off, ax_chunk_width(cols, OWt, VNt), s);
+            launch_cast_frag32(src, lds, rows, cols, transpose, m->d_mat32.p, off, ax_chunk_width(cols, ow, VNt), s);
         else if (tiled)
             launch_cast_tiled(src, lds, rows, cols, transpose, m->prec, m->d_mat32.p, m->d_mat16.p, off,
-                              ax_chunk_width(cols, OWt, VNt), VNt, s);
+                              ax_chunk_width(cols, ow, VNt), VNt, s);
         else
             launch_cast_block(src, lds, rows, cols, transpose, m->prec, m->d_mat32.p, m->d_mat16.p, off, ld, s);
     };
@@ -1089,11 +1108,11 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
                                   ldH[d], s);
             }
         } else {
-            cast_ax(Xd, NI, ni, ni, 0, h_off[d], ldH[d]);
+            cast_ax(Xd, NI, ni, ni, 0, h_off[d], ldH[d], OWt);
         }
         if (nbd > 0) {
-            cast_ax(Pd, NBp, ni, nbd, 0, p_off[d], ldP[d]);
-            cast_ax(Pd, NBp, nbd, ni, 1, t_off[d], ldT[d]);
+            cast_ax(Pd, NBp, ni, nbd, 0, p_off[d], ldP[d], OWc);
+            cast_ax(Pd, NBp, nbd, ni, 1, t_off[d], ldT[d], OWb);
         }
     }
     // row-form blocks: row-major, or the BF16 fragment layout of the tensor cores
@@ -1131,9 +1150,9 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
         // t_d = K_ii^-1 b_i (needed only by the back-substitution)
         const int OW = ax_outputs_per_block(m->prec);
         // tiled descriptors: ld = the chunk width, one block per chunk
-        auto tile_desc = [&](AxDesc& a) {
+        auto tile_desc = [&](AxDesc& a, int ow) {
             if (!a.tiled) return OW;
-            a.ld = ax_chunk_width(a.n_out, OWt, VN);
+            a.ld = ax_chunk_width(a.n_out, ow, VN);
             return (int)a.ld;
         };
         std::vector<AxDesc> dc, di, db, dm1, dm2;
@@ -1152,7 +1171,7 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
             c.n_out = nbd;
             c.tiled = tiled ? 1 : 0;
             if (nbd > 0) {
-                const int cw = tile_desc(c);
+                const int cw = tile_desc(c, OWc);
                 for (int32_t o0 = 0; o0 < c.n_out; o0 += cw) bc.push_back(AxBlock{(int32_t)dc.size(), o0});
                 dc.push_back(c);
             }
@@ -1162,7 +1181,7 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
                 t.out_off = tc_off[d];
                 t.ld = ldH[d];
                 t.n_out = ni;
-                const int cw = tile_desc(t);
+                const int cw = tile_desc(t, OWt);
                 for (int32_t o0 = 0; o0 < t.n_out; o0 += cw) bi.push_back(AxBlock{(int32_t)di.size(), o0});
                 di.push_back(t);
             } else if (r_dom[d] > 0) {
@@ -1202,7 +1221,7 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
             b.ld = ldT[d];
             b.n_out = ni;
             b.tiled = tiled ? 1 : 0;
-            const int cwb = tile_desc(b);
+            const int cwb = tile_desc(b, OWb);
             for (int32_t o0 = 0; o0 < b.n_out; o0 += cwb) bb.push_back(AxBlock{(int32_t)db.size(), o0});
             db.push_back(b);
         }

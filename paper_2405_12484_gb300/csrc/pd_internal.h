@@ -524,6 +524,7 @@ struct pd_mesh {
     // materials (pd_set_materials): the adjoint workspace's FP64 state and
     // FP64 per-tet weights follow them
     uint64_t state_gen = 0, mat_gen = 0;
+    uint64_t factor_gen = 0;   // pd_prefactor calls: the solve's buffers and launches change with each
     // state flags
     bool materials_set = false;
     bool prefactored = false;
@@ -576,6 +577,19 @@ struct pd_adjoint {
     pdg::DBuf<float4> ent_part;
     pdg::DBuf<int32_t> ent_ptr, ent;
     pdg::DBuf<double> mp_part, php_part;
+    // two CG iterations as a graph, by the solution vector they advance (one of this workspace's), see adjoint_pcg
+    struct PcgGraph {
+        cudaGraphExec_t exec = nullptr;
+        int32_t solves = 0;
+    };
+    std::map<float4*, PcgGraph> pcg_graphs;
+    uint64_t pcg_gen = 0;              // factor_gen they belong to
+    void drop_pcg_graphs() {
+        for (auto& g : pcg_graphs)
+            if (g.second.exec) cudaGraphExecDestroy(g.second.exec);
+        pcg_graphs.clear();
+    }
+    ~pd_adjoint() { drop_pcg_graphs(); }
     pdg::DBuf<double> partial, sc;
     pdg::DBuf<float> vol;
     pdg::DBuf<int32_t> user_of_tet;
