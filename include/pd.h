@@ -53,7 +53,7 @@ enum {
     PD_ERR_BAD_MESH = -2,         /* index out of range, repeated corner, rest volume <= 0, isolated vertex */
     PD_ERR_BAD_MATERIAL = -3,     /* gamma < 0 or non-finite (Sec. 6: gamma >= 0) */
     PD_ERR_NOT_PREFACTORED = -4,  /* pd_step before pd_prefactor, or after pd_set_materials */
-    PD_ERR_NOT_SPD = -5,          /* a Cholesky pivot was <= 0 during pd_prefactor */
+    PD_ERR_NOT_SPD = -5,          /* a pivot of a factorised matrix was <= 0 during pd_prefactor */
     PD_ERR_NO_MEMORY = -6,        /* device or host allocation failed */
     PD_ERR_NONFINITE = -7,        /* NaN/Inf found in the state (device flag) */
     PD_ERR_TIMEOUT = -8,          /* a bounded wait expired */
@@ -97,7 +97,8 @@ enum {
 typedef struct pd_solver_opts {
     int32_t precision;     /* PD_PREC_*; default PD_PREC_FP32 */
     int32_t refine_steps;  /* 0..2 extra refinement steps per PD iteration with an FP64 residual r = b - K x */
-    int32_t use_graphs;    /* 1: replay each frame as a captured CUDA graph (default), 0: plain launches */
+    int32_t use_graphs;    /* 1: replay frames, and solves and CG iterations that recur, as captured
+                              CUDA graphs (default), 0: plain launches */
     int32_t flags;         /* PD_SOLVE_* bits; 0 = direct solve x = S(b) */
     int32_t modes;         /* PD_SOLVE_MODAL: normal modes per domain (1..64; 0 = 20) */
     int32_t jacobi_sweeps; /* PD_SOLVE_MODAL: Chebyshev-Jacobi sweeps after the subspace solve (0..1000) */
@@ -163,7 +164,7 @@ pd_status pd_set_materials(pd_mesh* mesh, const float* gamma_s, const float* gam
 /*
  * pd_prefactor -- assemble K = M/dt^2 + sum_e V_e (gs+gv) B^T (D^T:D) B
  * (Sec. 7.1) and precompute the subspace solve on the device in FP64
- * (Sec. 7.2): per domain the Cholesky factor of K_ii, K_ii^-1 and the
+ * (Sec. 7.2): per domain K_ii^-1 (by symmetric block sweeps) and the
  * boundary modes Psi = -K_ii^-1 K_ib (Eq. cms_boundary); the reduced
  * interface matrix S = K_BB + sum_d K_bi Psi and its inverse; then the
  * per-iteration copies in the requested precision.

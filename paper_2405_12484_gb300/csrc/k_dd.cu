@@ -362,9 +362,9 @@ __global__ void __launch_bounds__(32 * kAxWarps) k_axpy_form(const AxDesc* __res
 
 // The same product streamed through shared memory with bulk asynchronous
 // copies (tiled layout only): one producer lane copies the block's tile in
-// stages of kAxtRows rows (one cp.async.bulk per stage, a ring of kAxtStages
-// stages of kAxtRows x w elements, completion counted in bytes on an
-// mbarrier), so the copies in flight do not depend on what the compute
+// stages of R rows (a multiple of kAxtRows chosen by ax_stage_rows; one
+// cp.async.bulk per stage, a ring of kAxtStages stages of R x w elements,
+// completion counted in bytes on an mbarrier), so the copies in flight do not depend on what the compute
 // warps do.  kAxtWarps consumer warps take the rows of a stage in turn (row
 // r to warp r mod kAxtWarps), each lane owning VN consecutive outputs with
 // x_k a shared-memory broadcast; after the last stage the warps' partial
