@@ -73,9 +73,11 @@ def parse():
 # ("dd_interior", fp32, two levels): the ncu capture of the interior k_axpy_tma launch on the
 # 153,600-tet shell; the interior is one tile stream per domain, so the ratio carries over to the
 # full-size launch.
-# Thread instructions per tet and SIMT efficiency of the fused local step from its ncu capture
-# (profiles/k_local_assemble_shell153k_fp32.md): its roofline is the issue rate, not HBM.
-LOCAL_THREAD_INSTR_PER_TET, LOCAL_SIMT = 1052.0, 22.41
+# Warp instructions of the fused local step per tet from its ncu captures, by form (its roofline is the
+# issue rate, not HBM): direct with the SVD (1,052 thread instructions at 22.41 lanes,
+# profiles/k_local_assemble_shell153k_fp32.md), correction without (8.10M for 390K tets,
+# profiles/k_local_assemble_fast_shell390k.md).
+LOCAL_WARP_INSTR_PER_TET = {False: 1052.0 / 22.41, True: 8.10e6 / 390000}
 TRAFFIC_RATIO = {("dd_interior", "fp32", "two"): 0.9931, ("dd_interior", "bf16", "two"): 0.991}
 
 
@@ -609,12 +611,12 @@ def main():
         if ck == "local" and not args.small:
             # issue-rate roofline: warp instructions of the launch against 4 per SM and cycle at the SM clock
             sm_hz = (leg["clocks"].get("sm_max_mhz") or 2070.0) * 1e6
-            warp_instr = w.n_t * LOCAL_THREAD_INSTR_PER_TET / LOCAL_SIMT
+            warp_instr = w.n_t * LOCAL_WARP_INSTR_PER_TET[bool(args.correction)]
             peak_issue = torch.cuda.get_device_properties(local).multi_processor_count * 4 * sm_hz
             achieved_issue = warp_instr / (ph[ck]["ms"] * 1e-3)
             critical["alu"] = {"bound": "alu", "warp_instructions": warp_instr, "achieved": achieved_issue,
                                "peak": peak_issue, "unit": "warp instructions/s", "frac": achieved_issue / peak_issue,
-                               "source": "instructions per tet and SIMT efficiency of k_local_assemble from its ncu "
+                               "source": "warp instructions per tet of k_local_assemble from its ncu "
                                          "capture over the phase's time (which includes k_assemble_shared); "
                                          "peak = SMs x 4 schedulers x 1 instruction per cycle x SM clock"}
 

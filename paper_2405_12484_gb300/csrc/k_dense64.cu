@@ -275,8 +275,9 @@ __global__ void __launch_bounds__(kThr) k_gemm64(int M, int N, int KC, double al
 // tile and the panel (25 us); the tiles of a batch are bound by the tensor cores (36 products per FP64
 // product, mma.sync).  Measured against the blocked Cholesky factorisation and substitution on the FP64 pipe
 // that it replaces (GB300, events): n = 512 x 25 matrices 9.9 -> 1.06 ms, 512 x 200 50.0 -> 6.4 ms, 1472 x 8
-// 50.6 -> 4.7 ms, 1984 x 1 30.3 -> 3.1 ms, 2880 x 1 60.8 -> 4.6 ms; max |A X - I| 8e-14 .. 2e-12 (the old one
-// 3e-14 .. 1e-12), and dense_gemm's error against 64-bit-exact sums 4e-16 of sum |a||b| (2e-15 on the FP64 pipe).
+// 50.6 -> 4.7 ms, 1984 x 1 30.3 -> 3.1 ms, 2880 x 1 60.8 -> 4.6 ms; largest relative error of an entry of X
+// against columns refined in quadruple precision 1e-15 .. 4e-13 (the old one 9e-14 .. 8e-13; |A X - I| of the same
+// order for both), and dense_gemm's error against exact sums 4e-16 of sum |a||b| (2e-15 on the FP64 pipe).
 
 // Double-float arithmetic (pairs of floats, about 48 bits) for the pivot blocks: an FP64 instruction of a warp
 // occupies its quarter of the SM for about 60 clocks, these 15 FP32 ones for 15.  The intrinsics keep the
