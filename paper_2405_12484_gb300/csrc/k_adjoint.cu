@@ -193,21 +193,21 @@ __global__ void __launch_bounds__(128) k_hvp_local(int n_t, const int4* __restri
     store_corners(dP, T, force + 4 * (int64_t)e);
 }
 
-// ---- preconditioned CG: one iteration in four launches beside the solve
+// ---- preconditioned CG: one iteration in five launches beside the solve
 //
-// k_pcg_direction: beta = r.z / (r.z before), p = z + beta p, and the partial sums of m/dt^2 |p|^2
+// k_pcg_direction: beta = r.z / (r.z before), p = z + beta p
 // k_pcg_hvp:       per block of kLaTets tets (the plan of the local step) the per-vertex sums of d^2E[p]'s corner
-//                  forces, one per block-vertex entry, and the partial sums of (p at the vertex) . entry; p.Hp is the
-//                  two sums' total
-// k_pcg_update:    alpha = r.z / p.Hp, x += alpha p, r -= alpha (m/dt^2 p + the vertex's entries)
+//                  forces, one per block-vertex entry
+// k_pcg_product:   Hp = m/dt^2 p + the vertex's entries, rounded once, and the partial sums of p.Hp
+// k_pcg_update:    alpha = r.z / p.Hp, x += alpha p, r -= alpha Hp
 // (the solve)      z = K^-1 r
 // k_dot_partial:   partial sums of r.z
-// Every block of the first and third adds the partial sums itself, in the same fixed order: no separate final
-// reduction, no Hp vector and no corner-force array.  p.Hp has to be that of the Hp that r gets (the energy
-// sum_e dF : dP differs from it by the rounding of the corner sums, and the last Newton corrections came out fifty
-// times noisier with it): it is taken from the stored entries, whose sum k_pcg_update rounds once.  The SVDs of a tet are taken once per solve (k_hvp_terms).
-// 50K-tet slab, one iteration: 80 us with thirteen launches (an SVD per tet in each; 9.5 + 9.1 us for H p and 14 us of
-// dots and vector updates, ncu), 48 us so; bound by the latency of nine dependent kernels.
+// The first and fourth add the partial sums in every block, in the same fixed order: no separate final reduction, and
+// no corner-force array.  p.Hp has to be that of the rounded Hp that r gets: with the energy sum_e dF : dP, which
+// differs by the rounding of the corner sums, the last Newton corrections came out fifty times noisier, and with the
+// sum over the unrounded entries (one launch less) still eight times.  The SVDs of a tet are taken once per solve
+// (k_hvp_terms).  50K-tet slab, one iteration: 80 us with thirteen launches (an SVD per tet in each; 9.5 + 9.1 us for
+// H p and 14 us of dots and vector updates, ncu), 46 us so; bound by the latency of ten dependent kernels.
 
 // (a fixed order: threads stride the array, then a tree)
 __device__ __forceinline__ double block_sum64(double v, double* sm /* 33 */) {
@@ -228,11 +228,9 @@ __device__ __forceinline__ double block_sum64(double v, double* sm /* 33 */) {
     return t;
 }
 
-__device__ __forceinline__ double partials_sum(const double* __restrict__ p, int n, const double* __restrict__ p2, int n2,
-                                               double* sm) {
+__device__ __forceinline__ double partials_sum(const double* __restrict__ p, int n, double* sm) {
     double v = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) v += p[i];
-    for (int i = threadIdx.x; i < n2; i += blockDim.x) v += p2[i];
     return block_sum64(v, sm);
 }
 
@@ -264,33 +262,24 @@ __global__ void __launch_bounds__(128) k_hvp_terms(int n_t, const int4* __restri
 // sc[parity]: r.z of this iteration, sc[1 - parity]: of the one before
 __global__ void __launch_bounds__(256) k_pcg_direction(int n, const double* __restrict__ rz_part, int n_rz,
                                                        double* __restrict__ sc, int parity, int first,
-                                                       const float* __restrict__ mh2, const float4* __restrict__ z,
-                                                       float4* __restrict__ p, double* __restrict__ mp_part) {
+                                                       const float4* __restrict__ z, float4* __restrict__ p) {
     __shared__ double sm[33];
     pdl_trigger();
     const int i = blockIdx.x * 256 + threadIdx.x;
-    const float m = i < n ? mh2[i] : 0.f;
     pdl_wait();
     float4 zi = make_float4(0.f, 0.f, 0.f, 0.f), pi = zi;
     if (i < n) {               // (loads in flight during the reduction)
         zi = z[i];
         if (!first) pi = p[i];
     }
-    const double rz = partials_sum(rz_part, n_rz, nullptr, 0, sm);
+    const double rz = partials_sum(rz_part, n_rz, sm);
     float be = 0.f;
     if (!first) {
         const double old = sc[1 - parity];
         be = fabs(old) > 1e-300 ? (float)(rz / old) : 0.f;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) sc[parity] = rz;
-    double acc = 0.0;
-    if (i < n) {
-        const float4 q = make_float4(zi.x + be * pi.x, zi.y + be * pi.y, zi.z + be * pi.z, 0.f);
-        p[i] = q;
-        acc = (double)m * ((double)q.x * q.x + (double)q.y * q.y + (double)q.z * q.z);
-    }
-    acc = block_sum64(acc, sm);
-    if (threadIdx.x == 0) mp_part[blockIdx.x] = acc;
+    if (i < n) p[i] = make_float4(zi.x + be * pi.x, zi.y + be * pi.y, zi.z + be * pi.z, 0.f);
 }
 
 // s + e += a b with the rounding errors of both operations kept in e (Ogita, Rump, Oishi, "Accurate sum and dot
@@ -305,12 +294,10 @@ __device__ __forceinline__ void dot2_add(float a, float b, float& s, float& e) {
 __global__ void __launch_bounds__(PDG_LA_TETS) k_pcg_hvp(int n_t, const int4* __restrict__ tets,
                                                          const float4* __restrict__ geo, const float* __restrict__ hess,
                                                          const float4* __restrict__ p, const int* __restrict__ vptr,
-                                                         const int* __restrict__ vert, const int* __restrict__ cptr,
-                                                         const uint16_t* __restrict__ corner, float4* __restrict__ part,
-                                                         double* __restrict__ php_part) {
+                                                         const int* __restrict__ cptr,
+                                                         const uint16_t* __restrict__ corner, float4* __restrict__ part) {
     constexpr int B = PDG_LA_TETS;
     __shared__ float fx[4 * B], fy[4 * B], fz[4 * B];
-    __shared__ double sm[33];
     pdl_trigger();
     const int e = blockIdx.x * B + threadIdx.x, ec = min(e, n_t - 1);
     const Tet T = load_tet(ec, n_t, tets, geo);
@@ -342,9 +329,7 @@ __global__ void __launch_bounds__(PDG_LA_TETS) k_pcg_hvp(int n_t, const int4* __
         }
     }
     __syncthreads();
-    float s = 0.f, c = 0.f;
     for (int j = j0 + threadIdx.x; j < j1; j += B) {
-        const float4 pv = p[__ldg(&vert[j])];
         float ax = 0.f, ay = 0.f, az = 0.f;
         for (int k = __ldg(&cptr[j]); k < __ldg(&cptr[j + 1]); ++k) {
             const int q = __ldg(&corner[k]);
@@ -353,47 +338,60 @@ __global__ void __launch_bounds__(PDG_LA_TETS) k_pcg_hvp(int n_t, const int4* __
             az += fz[q];
         }
         part[j] = make_float4(ax, ay, az, 0.f);
-        dot2_add(pv.x, ax, s, c);
-        dot2_add(pv.y, ay, s, c);
-        dot2_add(pv.z, az, s, c);
     }
-    const double tot = block_sum64((double)s + (double)c, sm);
-    if (threadIdx.x == 0) php_part[blockIdx.x] = tot;
+}
+
+__global__ void __launch_bounds__(256) k_pcg_product(int n, const float* __restrict__ mh2,
+                                                     const int* __restrict__ ent_ptr, const int* __restrict__ ent,
+                                                     const float4* __restrict__ part, const float4* __restrict__ p,
+                                                     float4* __restrict__ Hp, double* __restrict__ php_part) {
+    __shared__ double sm[33];
+    pdl_trigger();
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    float m = 0.f;
+    int k0 = 0, k1 = 0;
+    if (i < n) {
+        m = mh2[i];
+        k0 = ent_ptr[i];
+        k1 = ent_ptr[i + 1];
+    }
+    pdl_wait();
+    double acc = 0.0;
+    if (i < n) {
+        const float4 pi = p[i];
+        float hx = 0.f, hy = 0.f, hz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;
+        dot2_add(m, pi.x, hx, cx);
+        dot2_add(m, pi.y, hy, cy);
+        dot2_add(m, pi.z, hz, cz);
+        for (int k = k0; k < k1; ++k) {
+            const float4 f = part[ent[k]];
+            dot2_add(1.f, f.x, hx, cx);
+            dot2_add(1.f, f.y, hy, cy);
+            dot2_add(1.f, f.z, hz, cz);
+        }
+        const float4 h = make_float4(hx + cx, hy + cy, hz + cz, 0.f);
+        Hp[i] = h;
+        acc = (double)pi.x * h.x + (double)pi.y * h.y + (double)pi.z * h.z;
+    }
+    acc = block_sum64(acc, sm);
+    if (threadIdx.x == 0) php_part[blockIdx.x] = acc;
 }
 
 __global__ void __launch_bounds__(256) k_pcg_update(int n, const double* __restrict__ sc, int parity,
-                                                    const double* __restrict__ mp_part, int n_mp,
                                                     const double* __restrict__ php_part, int n_php,
-                                                    const float* __restrict__ mh2, const int* __restrict__ ent_ptr,
-                                                    const int* __restrict__ ent, const float4* __restrict__ part,
-                                                    const float4* __restrict__ p, float4* __restrict__ x,
-                                                    float4* __restrict__ r) {
+                                                    const float4* __restrict__ p, const float4* __restrict__ Hp,
+                                                    float4* __restrict__ x, float4* __restrict__ r) {
     __shared__ double sm[33];
     pdl_trigger();
     const int i = blockIdx.x * 256 + threadIdx.x, ic = min(i, n - 1);
-    const float m = mh2[ic];
-    const int k0 = ent_ptr[ic], k1 = ent_ptr[ic + 1];
     pdl_wait();
-    const float4 pi = p[ic];   // (loads in flight during the reduction)
+    const float4 pi = p[ic], hi = Hp[ic];   // (loads in flight during the reduction)
     float4 xi = x[ic], ri = r[ic];
-    float hx = 0.f, hy = 0.f, hz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;
-    dot2_add(m, pi.x, hx, cx);
-    dot2_add(m, pi.y, hy, cy);
-    dot2_add(m, pi.z, hz, cz);
-    for (int k = k0; k < k1; ++k) {
-        const float4 f = part[ent[k]];
-        dot2_add(1.f, f.x, hx, cx);
-        dot2_add(1.f, f.y, hy, cy);
-        dot2_add(1.f, f.z, hz, cz);
-    }
-    hx += cx;
-    hy += cy;
-    hz += cz;
-    const double php = partials_sum(mp_part, n_mp, php_part, n_php, sm);
+    const double php = partials_sum(php_part, n_php, sm);
     const float al = fabs(php) > 1e-300 ? (float)(sc[parity] / php) : 0.f;
     if (i >= n) return;
     xi.x += al * pi.x; xi.y += al * pi.y; xi.z += al * pi.z;
-    ri.x -= al * hx; ri.y -= al * hy; ri.z -= al * hz;
+    ri.x -= al * hi.x; ri.y -= al * hi.y; ri.z -= al * hi.z;
     x[i] = xi;
     r[i] = ri;
 }
@@ -975,15 +973,17 @@ void launch_hvp_terms(const pd_mesh* m, const float4* x, float* hess, cudaStream
     PDG_CHECK_LAUNCH();
 }
 
-// The three launches of one iteration before the solve (see above): z, n_rz partial sums of r.z in, x and r advanced.
+// The four launches of one iteration before the solve (see above): z, n_rz partial sums of r.z in, x and r advanced.
 void launch_pcg_step(const pd_mesh* m, pd_adjoint* a, int n_rz, int iteration, float4* x, cudaStream_t s) {
     const int n = m->n_free, parity = iteration & 1, nv = pcg_vertex_blocks(n);
     launch_pdl(k_pcg_direction, dim3(nv), dim3(256), 0, s, n, a->partial.p, n_rz, a->sc.p, parity, iteration == 0,
-               m->d_mh2.p, a->z.p, a->p.p, a->mp_part.p);
+               a->z.p, a->p.p);
     launch_pdl(k_pcg_hvp, dim3(m->la_blocks), dim3(PDG_LA_TETS), 0, s, m->n_t, m->d_tets.p, m->d_geo.p, a->hess.p,
-               a->p.p, m->d_la_vptr.p, m->d_la_vert.p, m->d_la_cptr.p, m->d_la_corner.p, a->ent_part.p, a->php_part.p);
-    launch_pdl(k_pcg_update, dim3(nv), dim3(256), 0, s, n, a->sc.p, parity, a->mp_part.p, nv, a->php_part.p,
-               m->la_blocks, m->d_mh2.p, a->ent_ptr.p, a->ent.p, a->ent_part.p, a->p.p, x, a->r.p);
+               a->p.p, m->d_la_vptr.p, m->d_la_cptr.p, m->d_la_corner.p, a->ent_part.p);
+    launch_pdl(k_pcg_product, dim3(nv), dim3(256), 0, s, n, m->d_mh2.p, a->ent_ptr.p, a->ent.p, a->ent_part.p, a->p.p,
+               a->Hp.p, a->php_part.p);
+    launch_pdl(k_pcg_update, dim3(nv), dim3(256), 0, s, n, a->sc.p, parity, a->php_part.p, nv, a->p.p, a->Hp.p, x,
+               a->r.p);
     PDG_CHECK_LAUNCH();
 }
 

@@ -69,7 +69,7 @@ void adjoint_pcg(pd_mesh* m, pd_adjoint* a, const float4* x_lin, const float4* b
     };
     iteration(0, s);
     // From the third solve for this vector after a prefactorisation on, pairs of iterations (an odd and an even one)
-    // are replayed as a graph, which takes thirteen launches and four event calls an iteration from the host
+    // are replayed as a graph, which takes fourteen launches and four event calls an iteration from the host
     // (equilibrium and adjoint step of the 50K-tet slab: 8.1 ms with plain launches, 7.9 so).
     constexpr int kPlainSolves = 2;
     int k = 1;
@@ -177,7 +177,7 @@ pd_status pd_adjoint_create(pd_mesh* m, int32_t cg_iters, pd_adjoint** out) {
         a->cg_iters = cg_iters;
         const size_t nv = (size_t)m->n_v;
         DBuf<float4>* bufs[] = {&a->xeq, &a->vprev, &a->g, &a->rhs, &a->lam, &a->lam1, &a->lam2,
-                                &a->r, &a->z, &a->p, &a->dx};
+                                &a->r, &a->z, &a->p, &a->Hp, &a->dx};
         for (auto* b : bufs) {
             b->alloc(nv);
             PDG_CUDA(cudaMemsetAsync(b->p, 0, sizeof(float4) * nv, m->stream));
@@ -187,8 +187,7 @@ pd_status pd_adjoint_create(pd_mesh* m, int32_t cg_iters, pd_adjoint** out) {
         PDG_CUDA(cudaMemsetAsync(a->sc.p, 0, sizeof(double) * 8, m->stream));
         a->hess.alloc((size_t)hess_floats() * m->n_t);
         a->ent_part.alloc(m->la_entries);
-        a->mp_part.alloc(pcg_vertex_blocks(m->n_free));
-        a->php_part.alloc(std::max(m->la_blocks, 1));
+        a->php_part.alloc(pcg_vertex_blocks(m->n_free));
         // the local plan's block-vertex entries by vertex, in block order
         std::vector<int32_t> vert(m->la_entries), eptr(m->n_free + 1, 0), ent(m->la_entries);
         if (m->la_entries > 0)

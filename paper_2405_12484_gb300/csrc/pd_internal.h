@@ -570,13 +570,13 @@ struct pd_mesh {
 struct pd_adjoint {
     pd_mesh* mesh = nullptr;
     int32_t cg_iters = 30;
-    pdg::DBuf<float4> xeq, vprev, g, rhs, lam, lam1, lam2, r, z, p, dx;
+    pdg::DBuf<float4> xeq, vprev, g, rhs, lam, lam1, lam2, r, z, p, Hp, dx;
     // one CG iteration: per-tet Hessian terms, the sums of the local plan's block-vertex entries and the entries of
     // every free vertex, partial sums of the scalars
     pdg::DBuf<float> hess;
     pdg::DBuf<float4> ent_part;
     pdg::DBuf<int32_t> ent_ptr, ent;
-    pdg::DBuf<double> mp_part, php_part;
+    pdg::DBuf<double> php_part;
     // two CG iterations as a graph, by the solution vector they advance (one of this workspace's), see adjoint_pcg
     struct PcgGraph {
         cudaGraphExec_t exec = nullptr;
