@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(PDG_LA_TETS) k_pcg_hvp(int n_t, const int4* __
         H.be[k] = __ldg(h + (int64_t)(27 + k) * n_t);
     }
     const int j0 = __ldg(&vptr[blockIdx.x]), j1 = __ldg(&vptr[blockIdx.x + 1]);
-    pdl_wait();   // (the terms were written before the predecessor of this kernel's first launch ended)
+    pdl_wait();   // (the terms were complete before the solve's first iteration, see launch_pcg_step)
     float dF[3][3], dP[3][3];
     tet_grad(T, p, dF);
     hess_apply(H, T.ws + T.wv, dF, dP);
@@ -976,8 +976,12 @@ void launch_hvp_terms(const pd_mesh* m, const float4* x, float* hess, cudaStream
 // The four launches of one iteration before the solve (see above): z, n_rz partial sums of r.z in, x and r advanced.
 void launch_pcg_step(const pd_mesh* m, pd_adjoint* a, int n_rz, int iteration, float4* x, cudaStream_t s) {
     const int n = m->n_free, parity = iteration & 1, nv = pcg_vertex_blocks(n);
-    launch_pdl(k_pcg_direction, dim3(nv), dim3(256), 0, s, n, a->partial.p, n_rz, a->sc.p, parity, iteration == 0,
-               a->z.p, a->p.p);
+    // k_pcg_hvp reads the Hessian terms before its dependency wait: the first iteration starts only when everything
+    // before it, k_hvp_terms included, has completed (a plain launch), the later ones follow it
+    if (iteration == 0)
+        k_pcg_direction<<<nv, 256, 0, s>>>(n, a->partial.p, n_rz, a->sc.p, parity, 1, a->z.p, a->p.p);
+    else
+        launch_pdl(k_pcg_direction, dim3(nv), dim3(256), 0, s, n, a->partial.p, n_rz, a->sc.p, parity, 0, a->z.p, a->p.p);
     launch_pdl(k_pcg_hvp, dim3(m->la_blocks), dim3(PDG_LA_TETS), 0, s, m->n_t, m->d_tets.p, m->d_geo.p, a->hess.p,
                a->p.p, m->d_la_vptr.p, m->d_la_cptr.p, m->d_la_corner.p, a->ent_part.p);
     launch_pdl(k_pcg_product, dim3(nv), dim3(256), 0, s, n, m->d_mh2.p, a->ent_ptr.p, a->ent.p, a->ent_part.p, a->p.p,
