@@ -1532,14 +1532,13 @@ void launch_coarse(pd_mesh* m, const T* pool, const float4* cin, float4* part, c
 
 template <class T>
 int axt_smem_limit() {
-    static const int lim = std::min(allow_max_dynamic_smem(k_axpy_tma<T, false>),
-                                    allow_max_dynamic_smem(k_axpy_tma<T, true>));
-    return lim;
+    static PerDevice known;
+    return max_dynamic_smem(known, k_axpy_tma<T, false>, k_axpy_tma<T, true>);
 }
 
 int axm_smem_limit() {
-    static const int lim = std::min(allow_max_dynamic_smem(k_axpy_mma<false>), allow_max_dynamic_smem(k_axpy_mma<true>));
-    return lim;
+    static PerDevice known;
+    return max_dynamic_smem(known, k_axpy_mma<false>, k_axpy_mma<true>);
 }
 
 template <class T>
@@ -1873,8 +1872,8 @@ int rowdot_rows_per_unit(int prec) { return prec == PD_PREC_BF16 ? RowRows<__nv_
 bool rowdot_row_fits_stage(int ld, int elem_bytes) { return (int64_t)ld * elem_bytes <= kRowtStageBytes; }
 
 bool rowdot_mma_fits(int xcap) {
-    static const int optin_m = allow_max_dynamic_smem(k_rowdot_mma);
-    return rowm_smem_bytes(xcap) <= (size_t)optin_m;
+    static PerDevice known;
+    return rowm_smem_bytes(xcap) <= (size_t)max_dynamic_smem(known, k_rowdot_mma);
 }
 
 void build_row_plan(RowPlan& P, std::vector<RowDesc> descs, int prec, cudaStream_t s, bool mma) {

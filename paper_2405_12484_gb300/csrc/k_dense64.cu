@@ -613,9 +613,8 @@ struct Scratch {
 
 // the digit kernels' dynamic shared memory exceeds the default limit
 void allow_digit_smem() {
-    static const int lim = std::min(std::min(allow_max_dynamic_smem(k_gemm64), allow_max_dynamic_smem(k_sweep_first)),
-                                    std::min(allow_max_dynamic_smem(k_sweep_panel), allow_max_dynamic_smem(k_sweep_update)));
-    if (lim < kSmemDig) throw Fail{PD_ERR_UNSUPPORTED};
+    static PerDevice known;
+    if (max_dynamic_smem(known, k_gemm64, k_sweep_first, k_sweep_panel, k_sweep_update) < kSmemDig) throw Fail{PD_ERR_UNSUPPORTED};
 }
 
 constexpr int64_t kSplitBytes = 16 * (int64_t)kBlkVec + 4 * NB;   // digits and exponents of one 64 x 64 block

@@ -5,12 +5,15 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <climits>
 #include <string>
 #include <vector>
 #include <map>
 #include <memory>
 
 #include "../../include/pd.h"
+#include "per_device.h"
 
 namespace pdg {
 
@@ -46,6 +49,19 @@ inline int allow_max_dynamic_smem(K* kernel) {
     const int lim = optin - (int)fa.sharedSizeBytes;
     PDG_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
     return lim;
+}
+
+// The same for kernels that are launched often: the smallest of their limits, raised once on each device (the
+// attribute belongs to the current one).  `known`: a static of the caller.
+template <class... K>
+inline int max_dynamic_smem(PerDevice& known, K*... kernels) {
+    int dev = 0;
+    PDG_CUDA(cudaGetDevice(&dev));
+    return known.get(dev, [&] {
+        int lim = INT_MAX;
+        ((lim = std::min(lim, allow_max_dynamic_smem(kernels))), ...);
+        return lim;
+    });
 }
 
 // Programmatic dependent launch (sm_90 and later): a kernel launched with
