@@ -7,7 +7,7 @@
 // three-unknown problem of Eq. vol_pre with targets clamped to >= 0.01),
 // Eq. pd_local, Eq. energy (per-element gamma_s, gamma_v).  Ordinarily
 // strained elements get both targets as one isotropic function of F^T F;
-// inverted and strongly strained ones, and every one in the frames of the
+// inverted and strongly strained ones, and every one in pd_step's frames of the
 // direct form (see local_corners), by the SVD and the enumeration of the volume
 // problem's candidates (proj3.cuh).
 //
@@ -116,12 +116,17 @@ __device__ __noinline__ void svd_targets_rare(const float (&F)[3][3], float ws, 
 // c_i = w_s (1 - s_i) + w_v (d_i - s_i) (P = w_s (R - F) + w_v (V - F), the
 // elastic part of b - K x without cancellation: F = U diag(s) W^T).
 //
-// FAST: the SVD-free targets (strain_of).  The frames of the direct form (x =
-// S(b), FP32) do not use them: there the rounding of every local step enters
-// the positions at full size (an ulp of a 2 m garment is 4e-5 m/s of its
-// velocity), and their trajectories stay what they were.  In the
-// correction form it only enters the shrinking correction.  Frame of the 390K
-// shell with / without: BF16 1.57 / 1.67 ms (FP32 would gain 2.01 -> 1.98).
+// FAST: the SVD-free targets (strain_of).  pd_step's frames of the direct form
+// (x = S(b), FP32) do not use them: there the rounding of every local step
+// enters the positions at full size (an ulp of a 2 m garment is 4e-5 m/s of
+// its velocity), and their trajectories stay what they were.  In the
+// correction form it only enters the shrinking correction.  Served frames,
+// direct form too, use them: on one domain they were the stepper's bitwise
+// and are no longer, with the same error against FP64 (eight slabs and shells
+// of 1,008 to 50,700 elements, frames 1, 5 and 30: positions 2.1e-7 .. 1.0e-4
+// with, 2.1e-7 .. 1.4e-4 without; velocities 1.3e-5 .. 5.7e-3 and 1.4e-5 ..
+// 6.7e-3, the largest on the coarsest one-layer shell).  Six requests with /
+// without 42.8 / 46.0 ms, BF16 frame of the 390K shell 1.57 / 1.67 ms.
 template <bool RESID, bool FAST>
 __device__ __forceinline__ void local_corners(const LocalIn& L, float (&out)[4][3]) {
     const float e1[3] = {L.x1.x - L.x0.x, L.x1.y - L.x0.y, L.x1.z - L.x0.z};
