@@ -757,17 +757,6 @@ __global__ void __launch_bounds__(128) k_tet_stiffness(int n_t, const int4* __re
             o[a * (7 - a) / 2 + b] = w * (g[a][0] * g[b][0] + g[a][1] * g[b][1] + g[a][2] * g[b][2]);
 }
 
-// position of `c` in the ascending list col[lo, hi), or -1
-__device__ __forceinline__ int find_col(const int* __restrict__ col, int lo, int hi, int c) {
-    const int end = hi;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (col[mid] < c) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo < end && col[lo] == c ? lo : -1;
-}
-
 __global__ void __launch_bounds__(128) k_assemble_rows(int n_free, const int* __restrict__ inc_ptr,
                                                        const int* __restrict__ inc, const int4* __restrict__ tets,
                                                        const double* __restrict__ ke, const double* __restrict__ mass,
@@ -775,12 +764,13 @@ __global__ void __launch_bounds__(128) k_assemble_rows(int n_free, const int* __
                                                        const int* __restrict__ col, double* __restrict__ val,
                                                        const int* __restrict__ fptr, const int* __restrict__ fcol,
                                                        double* __restrict__ fval, float* __restrict__ fval32,
-                                                       float* __restrict__ mh2) {
+                                                       float* __restrict__ mh2, int* __restrict__ err) {
     const int i = blockIdx.x * 128 + threadIdx.x;
     if (i >= n_free) return;
     const int lo = ptr[i], hi = ptr[i + 1], flo = fptr[i], fhi = fptr[i + 1];
     for (int k = lo; k < hi; ++k) val[k] = 0.0;
     for (int k = flo; k < fhi; ++k) fval[k] = 0.0;
+    bool lost = false;
     for (int n = inc_ptr[i]; n < inc_ptr[i + 1]; ++n) {
         const int t = inc[n] >> 2, a = inc[n] & 3;
         const int4 q4 = tets[t];
@@ -793,26 +783,31 @@ __global__ void __launch_bounds__(128) k_assemble_rows(int n_free, const int* __
             if (q[b] < n_free) {
                 const int k = find_col(col, lo, hi, q[b]);
                 if (k >= 0) val[k] += v;
+                else lost = true;
             } else {
                 const int k = find_col(fcol, flo, fhi, q[b] - n_free);
                 if (k >= 0) fval[k] += v;
+                else lost = true;
             }
         }
     }
     const int d = find_col(col, lo, hi, i);
     const double m = mass[i] * inv_h2;
     if (d >= 0) val[d] += m;
+    else lost = true;
+    if (lost) atomicOr(err, ERR_NO_PLACE);
     mh2[i] = (float)m;
     for (int k = flo; k < fhi; ++k) fval32[k] = (float)fval[k];
 }
 
 // Dense K_ii (identity beyond the domain's rows) and K_ib of every domain from the rows of K (both zeroed before):
-// dom = (first internal vertex, count, offset and count of the boundary list) of a domain.
+// dom = (first internal vertex, count, offset and count of the boundary list) of a domain.  An entry without a place
+// sets ERR_NO_PLACE.
 __global__ void __launch_bounds__(128) k_domain_blocks(const int4* __restrict__ dom, const int* __restrict__ bnd,
                                                        int n_int, const int* __restrict__ ptr,
                                                        const int* __restrict__ col, const double* __restrict__ val,
                                                        double* __restrict__ Kii, int NI, double* __restrict__ Kib,
-                                                       int NBp) {
+                                                       int NBp, int* __restrict__ err) {
     const int r = blockIdx.x * 128 + threadIdx.x;
     if (r >= NI) return;
     const int4 D = dom[blockIdx.y];
@@ -823,13 +818,10 @@ __global__ void __launch_bounds__(128) k_domain_blocks(const int4* __restrict__ 
     }
     double* ib = Kib + ((int64_t)blockIdx.y * NI + r) * NBp;
     for (int k = ptr[D.x + r]; k < ptr[D.x + r + 1]; ++k) {
-        const int c = col[k];
-        if (c >= D.x && c < D.x + D.y) {
-            ii[c - D.x] = val[k];
-        } else if (c >= n_int) {
-            const int p = find_col(bnd, D.z, D.z + D.w, c - n_int);
-            if (p >= 0) ib[p - D.z] = val[k];
-        }
+        const int p = domain_place(col[k], D.x, D.y, bnd, D.z, D.w, n_int);
+        if (p < 0) atomicOr(err, ERR_NO_PLACE);
+        else if (p < D.y) ii[p] = val[k];
+        else ib[p - D.y] = val[k];
     }
 }
 
@@ -970,7 +962,7 @@ void launch_assemble_K(pd_mesh* m, double inv_h2, cudaStream_t s) {
     PDG_CHECK_LAUNCH();
     k_assemble_rows<<<(m->n_free + 127) / 128, 128, 0, s>>>(
         m->n_free, m->d_inc_ptr.p, m->d_inc.p, m->d_tets.p, ke.p, m->d_mass64.p, inv_h2, m->d_K_ptr.p, m->d_K_col.p,
-        m->d_K_val.p, m->d_kfp_ptr.p, m->d_kfp_col.p, fval.p, m->d_kfp_val.p, m->d_mh2.p);
+        m->d_K_val.p, m->d_kfp_ptr.p, m->d_kfp_col.p, fval.p, m->d_kfp_val.p, m->d_mh2.p, m->d_err.p);
     PDG_CHECK_LAUNCH();   // (the temporaries' release is stream-ordered, or waits for the device)
 }
 
@@ -978,7 +970,7 @@ void launch_domain_blocks(const pd_mesh* m, const int4* dom, const int* bnd, dou
                           cudaStream_t s) {
     if (m->n_dom <= 0) return;
     k_domain_blocks<<<dim3((NI + 127) / 128, m->n_dom), 128, 0, s>>>(dom, bnd, m->n_int, m->d_K_ptr.p, m->d_K_col.p,
-                                                                    m->d_K_val.p, Kii, NI, Kib, NBp);
+                                                                    m->d_K_val.p, Kii, NI, Kib, NBp, m->d_err.p);
     PDG_CHECK_LAUNCH();
 }
 

@@ -757,6 +757,7 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
     const double inv_h2 = 1.0 / (dt * dt);
 
     // ---- scalar K over free vertices, the free-pinned block and m / dt^2 (FP64, device, fixed order)
+    PDG_CUDA(cudaMemsetAsync(m->d_err.p, 0, sizeof(int32_t), s));
     launch_assemble_K(m, inv_h2, s);
 
     // ---- per-domain dense blocks K_ii (padded with identity) and K_ib
@@ -790,7 +791,6 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
     dXii.alloc((size_t)n_dom * sKii);
     dPsi.alloc((size_t)n_dom * sKib);
     dSd.alloc((size_t)n_dom * sSd);
-    PDG_CUDA(cudaMemsetAsync(m->d_err.p, 0, sizeof(int32_t), s));
     dense_spd_inverse(dKii.p, NI, NI, sKii, dXii.p, NI, sKii, n_dom, m->d_err.p, s);
     // Psi = -K_ii^-1 K_ib ;  S_d = K_ib^T Psi = -K_bi K_ii^-1 K_ib
     dense_gemm(false, false, NI, NBp, NI, -1.0, dXii.p, NI, sKii, dKib.p, NBp, sKib, 0.0, dPsi.p, NBp, sKib, n_dom, s);
@@ -1647,9 +1647,12 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
     int32_t herr = 0;
     PDG_CUDA(cudaMemcpyAsync(&herr, m->d_err.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     PDG_CUDA(cudaStreamSynchronize(s));
-    if (herr & ERR_NOT_SPD) {
+    if (herr & (ERR_NOT_SPD | ERR_NO_PLACE)) {
         PDG_CUDA(cudaMemsetAsync(m->d_err.p, 0, sizeof(int32_t), s));
         PDG_CUDA(cudaStreamSynchronize(s));
+        // (without all entries the pivots mean nothing)
+        if (herr & ERR_NO_PLACE)
+            return fail(PD_ERR_BAD_MESH, "internal vertex coupled to another domain's internal vertex");
         return fail(PD_ERR_NOT_SPD, "a Cholesky pivot was not positive");
     }
     // load the fixed scratch array of pd_solve_noalloc on this device now,

@@ -13,6 +13,7 @@
 #include <memory>
 
 #include "../../include/pd.h"
+#include "domain_rows.h"
 #include "per_device.h"
 
 namespace pdg {
@@ -89,7 +90,7 @@ inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 }
 
 // Device error flag bits (d_err).
-enum : int { ERR_NONFINITE = 1, ERR_NOT_SPD = 2, ERR_TIMEOUT = 4 };
+enum : int { ERR_NONFINITE = 1, ERR_NOT_SPD = 2, ERR_TIMEOUT = 4, ERR_NO_PLACE = 8 };
 
 // ---------------------------------------------------------------- device buffer
 // Allocation stream of the calling thread (set by AllocStreamScope): buffers
