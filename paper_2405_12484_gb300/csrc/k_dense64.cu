@@ -271,13 +271,18 @@ __global__ void __launch_bounds__(kThr) k_gemm64(int M, int N, int KC, double al
 // launches per 64 columns: k_sweep_panel forms W = C P (and the digits of C
 // and W), k_sweep_update forms B - W C^T on the lower tiles; its first block
 // per matrix also inverts the next pivot while the others update.
+// W = C P with P rounded to FP64 is not as good as a triangular solve where C P C^T cancels; there the panel refines
+// it (see cancels and refine_panel).  Errors max |X - X*| / max |X*| against extended precision, blocked Cholesky on the
+// FP64 pipe / plain sweeps / these: lattices of 400 vertices moved by up to 45 % of an edge, two decades of stiffness,
+// dt = 1 s 1.6e-8 / 1.3e-7 / 1.2e-9; I + v v^T with a condition of 2^20 over two pivots 2.0e-11 / 1.1e-6 / 7.1e-12; regular
+// lattices, two decades, dt = 1/150 s 1.7e-15 / 2.3e-15 / 2.3e-15 (not refined).
 // What bounds it: one matrix is a chain of n / 64 steps, each the pivot's inversion on one SM (about 60 us), its
 // tile and the panel (25 us); the tiles of a batch are bound by the tensor cores (36 products per FP64
 // product, mma.sync).  Measured against the blocked Cholesky factorisation and substitution on the FP64 pipe
 // that it replaces (GB300, events): n = 512 x 25 matrices 9.9 -> 1.06 ms, 512 x 200 50.0 -> 6.4 ms, 1472 x 8
-// 50.6 -> 4.7 ms, 1984 x 1 30.3 -> 3.1 ms, 2880 x 1 60.8 -> 4.6 ms; largest relative error of an entry of X
-// against columns refined in quadruple precision 1e-15 .. 4e-13 (the old one 9e-14 .. 8e-13; |A X - I| of the same
-// order for both), and dense_gemm's error against exact sums 4e-16 of sum |a||b| (2e-15 on the FP64 pipe).
+// 50.6 -> 4.7 ms, 1984 x 1 30.3 -> 3.1 ms, 2880 x 1 60.8 -> 4.6 ms (the choice of refinement is 1 % of these);
+// dense_gemm's error against exact sums 4e-16 of sum |a||b| on rows of ordinary range (2e-15 on the FP64 pipe), 2^-60 of
+// the row maxima's product for entries far below the maximum of their row of 64.
 
 // Double-float arithmetic (pairs of floats, about 48 bits) for the pivot blocks: an FP64 instruction of a warp
 // occupies its quarter of the SM for about 60 clocks, these 15 FP32 ones for 15.  The intrinsics keep the
@@ -307,6 +312,7 @@ __device__ __forceinline__ DF df_fnma(DF a, DF b, DF c) {
     return {s, __fadd_rn(e, __fsub_rn(c.l, l))};
 }
 
+// (a __grid_constant__ parameter: its address goes to the routines out of line without a copy on the stack)
 struct SweepArgs {
     double* A;             // the matrix (lower tiles), swept in place
     int lda, nblk;         // row stride, n / 64
@@ -314,6 +320,9 @@ struct SweepArgs {
     double* P;             // per matrix: 64 x 64 inverse of the pivot, then its digits
     uint4* dP;
     int* eP;
+    uint4* dD;             // per matrix: digits of the scaled pivot D' = S D S, S = 2^-ex; eD: their exponents + ex
+    int *eD, *ex;
+    float *sx, *nu;        // per matrix: square roots of the diagonal of X = D'^-1, its largest -X_kj / (sx_k sx_j)
     uint4 *dC, *dW;        // per matrix: digits of the panel C and of W, nblk blocks each
     int *eC, *eW;
     int* err;
@@ -322,6 +331,8 @@ struct SweepArgs {
 struct PivotSmem {
     int es[NB], es2[NB], ex[NB];
     DF col[2][NB];
+    float sx[NB];
+    unsigned nu;
     int bad;
 };
 
@@ -334,7 +345,10 @@ struct PivotSmem {
 //   P  = S X S
 __device__ __noinline__ void finish_pivot(const SweepArgs& S, int z, double (*sm)[NB + 1], uint4* dsm, PivotSmem& T) {
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    if (threadIdx.x == 0) T.bad = 0;
+    if (threadIdx.x == 0) {
+        T.bad = 0;
+        T.nu = 0;
+    }
     __syncthreads();
     if (threadIdx.x < NB) {
         const double d = sm[threadIdx.x][threadIdx.x];
@@ -415,9 +429,25 @@ __device__ __noinline__ void finish_pivot(const SweepArgs& S, int z, double (*sm
                 sm[r][c] = v;
                 sm[c][r] = v;
             }
+            if (r == c) T.sx[r] = sqrtf(fmaxf(-m[a][b].h, 0.f));
         }
     __syncthreads();
     uint4 *dD = dsm, *dX = dsm + kBlkVec;
+    // for the panel's choice and its refinement (see k_sweep_panel)
+    float nu = 0.f;
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2 * a + 2; ++b)
+            if (ty + 32 * a > tx + 16 * b) nu = fmaxf(nu, __fdividef(m[a][b].h, T.sx[ty + 32 * a] * T.sx[tx + 16 * b]));
+    const unsigned wnu = __reduce_max_sync(0xffffffffu, __float_as_uint(nu));
+    if ((threadIdx.x & 31) == 0) atomicMax(&T.nu, wnu);
+    for (int l = threadIdx.x; l < kBlkVec; l += kThr) S.dD[(int64_t)z * kBlkVec + l] = dD[l];
+    if (threadIdx.x < NB) {
+        S.eD[z * NB + threadIdx.x] = T.es[threadIdx.x] + T.ex[threadIdx.x];
+        S.ex[z * NB + threadIdx.x] = T.ex[threadIdx.x];
+        S.sx[z * NB + threadIdx.x] = T.sx[threadIdx.x];
+    }
     split_block(sm, T.es2, dX);
     double x[2][4];
 #pragma unroll
@@ -453,10 +483,13 @@ __device__ __noinline__ void finish_pivot(const SweepArgs& S, int z, double (*sm
     store_digits(S.dP + (int64_t)z * kBlkVec, dD, S.eP + z * NB, T.es);
     double* P = S.P + (int64_t)z * NB * NB;
     for (int l = threadIdx.x; l < NB * NB; l += kThr) P[l] = sm[l / NB][l % NB];
-    if (threadIdx.x == 0 && T.bad) atomicOr(S.err, ERR_NOT_SPD);
+    if (threadIdx.x == 0) {
+        S.nu[z] = __uint_as_float(T.nu);
+        if (T.bad) atomicOr(S.err, ERR_NOT_SPD);
+    }
 }
 
-__global__ void __launch_bounds__(kThr) k_sweep_first(SweepArgs S) {
+__global__ void __launch_bounds__(kThr) k_sweep_first(const __grid_constant__ SweepArgs S) {
     extern __shared__ uint4 dsm[];
     __shared__ double sm[NB][NB + 1];
     __shared__ PivotSmem T;
@@ -465,8 +498,86 @@ __global__ void __launch_bounds__(kThr) k_sweep_first(SweepArgs S) {
     finish_pivot(S, blockIdx.x, sm, dsm, T);
 }
 
+// x 2^-e to 20 bits (zero below 2^-100, infinite above 2^100)
+__device__ __forceinline__ float coarse(double x, int e) {
+    const int hi = __double2hiint(x), f = ((hi >> 20) & 0x7ff) - 1023 - e;
+    const unsigned sign = (unsigned)hi & 0x80000000u;
+    if (f < -100) return 0.f;
+    if (f > 100) return __uint_as_float(sign | 0x7f800000u);
+    return __uint_as_float(sign | (unsigned)(f + 127) << 23 | ((unsigned)hi & 0xfffffu) << 3);
+}
+
+// Whether W = C P of the row block in sm needs the refinement: P is rounded to FP64, so W C^T is off by up to
+// u |C| P |C|^T, where a Cholesky factorisation is off by u times the diagonal of B.  The first is C P C^T (at most
+// that diagonal) where nothing cancels, as in the M-matrices of well-shaped elements (C <= 0 <= P); in general it is
+// at most C P C^T + 4 t+ t- + 2 nu t^2 with t+- = sum_k (C_ik)+- P_kk^1/2, t their sum, and nu the most negative entry of
+// P relative to its diagonal.  Refine where the added terms exceed twice the diagonal: never on the lattices of the
+// slabs and shells (largest measured 0.7), on about half of the row blocks of lattices with vertices moved by up to 30 or 45 %.
+__device__ __forceinline__ bool cancels(const SweepArgs& S, int z, int i, const double (*sm)[NB + 1]) {
+    const int r = threadIdx.x >> 3;
+    const double* A = S.A + (int64_t)z * S.sA;
+    const double d = A[(int64_t)(i * NB + r) * (S.lda + 1)];
+    const int e = (exponent_field(d) - 1023) >> 1;
+    float tp = 0.f, tm = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int c = (threadIdx.x & 7) + 8 * k;
+        const float v = coarse(sm[r][c], S.ex[z * NB + c] + e) * S.sx[z * NB + c];
+        tp += fmaxf(v, 0.f);
+        tm += fmaxf(-v, 0.f);
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        tp += __shfl_xor_sync(0xffffffffu, tp, o);
+        tm += __shfl_xor_sync(0xffffffffu, tm, o);
+    }
+    const float t = tp + tm;
+    return !(4.f * tp * tm + 2.f * S.nu[z] * t * t <= 2.f * fabsf(coarse(d, 2 * e)));
+}
+
+// W += (C - W D) P with exact products: W D is C to rounding then, as with a triangular solve.  T: the tile of C
+// (transposed if flip); sC, sP: digits, sP those of P on entry and exit.
+__device__ __noinline__ void refine_panel(const SweepArgs& S, int z, const double* T, bool flip, double (*sm)[NB + 1],
+                                          int* es, uint4* sC, uint4* sP, double (&w)[2][4]) {
+    float acc[kDig][2][4];
+    const uint4 *dP = S.dP + (int64_t)z * kBlkVec, *dD = S.dD + (int64_t)z * kBlkVec;
+    __syncthreads();           // es and the digits in sC and sP are read
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sm[tile_row(e)][tile_col(q, e)] = scale2(w[q][e], S.ex[z * NB + tile_col(q, e)]);
+    for (int l = threadIdx.x; l < kBlkVec; l += kThr) sP[l] = dD[l];
+    __syncthreads();
+    split_block(sm, es, sC);   // W S^-1, so that W D = (W S^-1) D' S^-1
+    __syncthreads();
+    mma_block<false>(sC, sP, acc);
+    double res[2][4];
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int r = tile_row(e), c = tile_col(q, e);
+            res[q][e] = T[flip ? (int64_t)c * S.lda + r : (int64_t)r * S.lda + c] -
+                        combine(acc, q, e, es[r] + S.eD[z * NB + c]);
+        }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sm[tile_row(e)][tile_col(q, e)] = res[q][e];
+    for (int l = threadIdx.x; l < kBlkVec; l += kThr) sP[l] = dP[l];
+    __syncthreads();
+    split_block(sm, es, sC);
+    __syncthreads();
+    mma_block<false>(sC, sP, acc);
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) w[q][e] += combine(acc, q, e, es[tile_row(e)] + S.eP[z * NB + tile_col(q, e)]);
+}
+
 // Row block blockIdx.y of matrix blockIdx.x: C_i, W_i = C_i P into the matrix, the digits of both.
-__global__ void __launch_bounds__(kThr) k_sweep_panel(SweepArgs S, int k) {
+__global__ void __launch_bounds__(kThr) k_sweep_panel(const __grid_constant__ SweepArgs S, int k) {
     extern __shared__ uint4 dsm[];
     __shared__ double sm[NB][NB + 1];
     __shared__ int es[NB];
@@ -489,8 +600,9 @@ __global__ void __launch_bounds__(kThr) k_sweep_panel(SweepArgs S, int k) {
     uint4 *sC = dsm, *sP = dsm + kBlkVec;
     const uint4* dP = S.dP + (int64_t)z * kBlkVec;
     for (int l = threadIdx.x; l < kBlkVec; l += kThr) sP[l] = dP[l];
+    const bool own = cancels(S, z, i, sm);
     split_block(sm, es, sC);
-    __syncthreads();
+    const bool refine = __syncthreads_or(own) != 0;
     store_digits(S.dC + blk * kBlkVec, sC, S.eC + blk * NB, es);
     float acc[kDig][2][4];
     mma_block<false>(sC, sP, acc);
@@ -500,6 +612,12 @@ __global__ void __launch_bounds__(kThr) k_sweep_panel(SweepArgs S, int k) {
 #pragma unroll
         for (int e = 0; e < 4; ++e)
             w[q][e] = combine(acc, q, e, es[tile_row(e)] + S.eP[z * NB + tile_col(q, e)]);
+    if (refine) {
+        double v[2][4];        // (w stays in registers)
+        memcpy(v, w, sizeof(v));
+        refine_panel(S, z, T, flip, sm, es, sC, sP, v);
+        memcpy(w, v, sizeof(v));
+    }
     __syncthreads();           // es and the digits of C are rewritten below
 #pragma unroll
     for (int q = 0; q < 2; ++q)
@@ -515,7 +633,7 @@ __global__ void __launch_bounds__(kThr) k_sweep_panel(SweepArgs S, int k) {
 
 // Lower tile (i, j), i, j != k, of one matrix: B_ij -= W_i C_j^T.  Tile 0 is the next pivot (k + 1, k + 1), which its
 // block then inverts (all matrices' first, so that the long blocks start first); the others follow row by row.
-__global__ void __launch_bounds__(kThr) k_sweep_update(SweepArgs S, int k, int batch) {
+__global__ void __launch_bounds__(kThr) k_sweep_update(const __grid_constant__ SweepArgs S, int k, int batch) {
     extern __shared__ uint4 dsm[];
     __shared__ double sm[NB][NB + 1];
     __shared__ PivotSmem ps;
@@ -672,21 +790,27 @@ void dense_spd_inverse(double* A, int n, int lda, int64_t sA, double* X, int ldx
     if (n <= 0 || batch <= 0) return;
     allow_digit_smem();
     const int nblk = n / NB;
-    const int zb = (int)std::max<int64_t>(1, std::min<int64_t>(batch, kScratchMax / (kSplitBytes * (2 * nblk + 1))));
+    const int zb = (int)std::max<int64_t>(1, std::min<int64_t>(batch, kScratchMax / (kSplitBytes * (2 * nblk + 2))));
     const int64_t nP = zb, nC = (int64_t)zb * nblk;
-    Scratch w((size_t)(kSplitBytes * (nP + 2 * nC) + sizeof(double) * NB * NB * nP), s);
+    constexpr int64_t kPivotBytes = sizeof(double) * NB * NB + 4 * (2 * NB + 1);   // P, ex, sx and nu
+    Scratch w((size_t)(kSplitBytes * (2 * nP + 2 * nC) + kPivotBytes * nP), s);
     SweepArgs S{};
     S.lda = lda;
     S.nblk = nblk;
     S.sA = sA;
     S.err = d_err;
     S.dP = static_cast<uint4*>(w.p);
-    S.dC = S.dP + nP * kBlkVec;
+    S.dD = S.dP + nP * kBlkVec;
+    S.dC = S.dD + nP * kBlkVec;
     S.dW = S.dC + nC * kBlkVec;
     S.P = reinterpret_cast<double*>(S.dW + nC * kBlkVec);
     S.eP = reinterpret_cast<int*>(S.P + nP * NB * NB);
-    S.eC = S.eP + nP * NB;
+    S.eD = S.eP + nP * NB;
+    S.ex = S.eD + nP * NB;
+    S.eC = S.ex + nP * NB;
     S.eW = S.eC + nC * NB;
+    S.sx = reinterpret_cast<float*>(S.eW + nC * NB);
+    S.nu = S.sx + nP * NB;
     for (int z0 = 0; z0 < batch; z0 += zb) {
         const int nz = std::min(zb, batch - z0);
         S.A = A + z0 * sA;
@@ -707,7 +831,7 @@ void dense_spd_inverse(double* A, int n, int lda, int64_t sA, double* X, int ldx
 
 int64_t dense_scratch_bytes(int n, int batch) {
     const int64_t nblk = (n + NB - 1) / NB;
-    const int64_t inv = kSplitBytes * (2 * nblk + 1), prod = 2 * kSplitBytes * nblk * nblk;
+    const int64_t inv = kSplitBytes * (2 * nblk + 2), prod = 2 * kSplitBytes * nblk * nblk;
     return std::max(inv, std::min<int64_t>(kScratchMax, std::max(inv, prod) * std::max(batch, 1)));
 }
 
