@@ -224,6 +224,9 @@ pd_status pd_project(const float* F, int32_t n, float* R, float* V, float* sigma
  * target y (both [device] n_v x 3): b = (M/dt^2) y + sum_e V_e B^T D^T :
  * (gs R + gv V) - K_fp x_p for free vertices (Sec. 7.1, b); rows of pinned
  * vertices are set to 0.  b [device] n_v x 3.  Requires pd_prefactor.
+ * Ordinarily strained elements get R and V without an SVD, as in pd_project,
+ * served frames and the correction form; pd_step's frames of the direct form
+ * take the SVD for every element, which differs by FP32 rounding.
  */
 pd_status pd_local_rhs(pd_mesh* mesh, const float* x, const float* y, float* b);
 

@@ -973,7 +973,8 @@ void launch_hvp_terms(const pd_mesh* m, const float4* x, float* hess, cudaStream
     PDG_CHECK_LAUNCH();
 }
 
-// The four launches of one iteration before the solve (see above): z, n_rz partial sums of r.z in, x and r advanced.
+// Four of the five launches of an iteration (see above; the fifth is k_dot_partial behind the solve): z and n_rz partial
+// sums of r.z in, x and r advanced.
 void launch_pcg_step(const pd_mesh* m, pd_adjoint* a, int n_rz, int iteration, float4* x, cudaStream_t s) {
     const int n = m->n_free, parity = iteration & 1, nv = pcg_vertex_blocks(n);
     // k_pcg_hvp reads the Hessian terms before its dependency wait: the first iteration starts only when everything

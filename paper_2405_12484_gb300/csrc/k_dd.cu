@@ -576,10 +576,14 @@ inline size_t axm_ring_bytes(int wmax, bool tf32, int stage_rows) {
 
 // Rows per stage of a launch (a multiple of `unit`; the results do not depend on it).  With many blocks per SM the
 // short stages of `unit` rows keep enough copies in flight; with less than two, a block alone waits for the latency of
-// each round of three stages (a 455-row tile in fifteen stages of 32 rows), so the stages grow to 64 KB a ring.
+// each round of three stages (a 455-row tile in fifteen stages of 32 rows), so the stages grow to 64 KB a ring.  Beside
+// that ring x and the A operands of the longest product that pd_create_mesh admits (kMaxSubCols rows: 16 bytes a row and up to 24)
+// fit in a block's shared memory.
+constexpr int kAxRingBytes = 65536;
+static_assert(kAxRingBytes + kMaxSubCols * (16 + 16 * kAxmFragLanes / 8) <= 224 * 1024, "the longest product fits");
 inline int ax_stage_rows(int n_blocks, int sms, int k_max, int w_max, int elem, int unit) {
     if (n_blocks >= 2 * sms) return unit;
-    const int fit = 65536 / (kAxtStages * std::max(w_max, 1) * elem) / unit * unit;
+    const int fit = kAxRingBytes / (kAxtStages * std::max(w_max, 1) * elem) / unit * unit;
     return std::max(unit, std::min(fit, (k_max + unit - 1) / unit * unit));
 }
 
@@ -1647,8 +1651,8 @@ void dd_solve_stream(pd_mesh* m, const float4* b, float4* xout, const DDBufs& w,
 // One product's arrays and launch properties.
 //   once: the per-domain matrices and S_II^-1 are most of an iteration's bytes (253 of 398 MB on the 390K shell, FP32)
 //     and return only in the next iteration; leaving L2 first, they keep the interface chain's matrices in it (129
-//     MB).  Frames measured without / with: 140K-tet shell FP32 1.07 / 0.94 ms, 390K BF16 1.65 / 1.59, 390K FP32 2.00 /
-//     1.98; no difference where everything fits (53K-tet shell).
+//     MB).  Frames without / with: 140K-tet shell FP32 1.14 / 1.00 ms, 390K BF16 1.68 / 1.62, 390K FP32 2.13 / 2.10;
+//     where everything fits nothing is gained (53K-tet shell TF32 574 / 578 us, FP32 520 / 523).
 //   late: see dd_solve_impl.
 AxBases product(const void* pool, const float4* x, const int* bidx, const float4* add, float4* out, bool once, bool late) {
     AxBases B{pool, x, bidx, add, out};

@@ -126,7 +126,9 @@ __device__ __noinline__ void svd_targets_rare(const float (&F)[3][3], float ws, 
 // of 1,008 to 50,700 elements, frames 1, 5 and 30: positions 2.1e-7 .. 1.0e-4
 // with, 2.1e-7 .. 1.4e-4 without; velocities 1.3e-5 .. 5.7e-3 and 1.4e-5 ..
 // 6.7e-3, the largest on the coarsest one-layer shell).  Six requests with /
-// without 42.8 / 46.0 ms, BF16 frame of the 390K shell 1.57 / 1.67 ms.
+// without 42.8 / 46.0 ms; BF16 frame of the 390K shell 1.57 / 1.67 ms; FP32
+// frames would gain from it: 390K shell 2.10 -> 2.00 ms, 140K shell 1.00 -> 0.93,
+// 10 iterations of the small slab 178 -> 164 us.
 template <bool RESID, bool FAST>
 __device__ __forceinline__ void local_corners(const LocalIn& L, float (&out)[4][3]) {
     const float e1[3] = {L.x1.x - L.x0.x, L.x1.y - L.x0.y, L.x1.z - L.x0.z};

@@ -1653,7 +1653,7 @@ pd_status pd_prefactor(pd_mesh* m, double dt, const pd_solver_opts* opts) {
         // (without all entries the pivots mean nothing)
         if (herr & ERR_NO_PLACE)
             return fail(PD_ERR_BAD_MESH, "internal vertex coupled to another domain's internal vertex");
-        return fail(PD_ERR_NOT_SPD, "a Cholesky pivot was not positive");
+        return fail(PD_ERR_NOT_SPD, "a pivot of a factorised matrix was not positive");
     }
     // load the fixed scratch array of pd_solve_noalloc on this device now,
     // while allocation is allowed (the runtime loads device modules lazily)
@@ -1812,7 +1812,7 @@ pd_status pd_sync(pd_mesh* m) {
             return fail(PD_ERR_TIMEOUT, "a pipeline wait in the subspace solve ran out");
         }
         if (herr & ERR_NONFINITE) return fail(PD_ERR_NONFINITE, "non-finite positions or velocities");
-        return fail(PD_ERR_NOT_SPD, "a Cholesky pivot was not positive");
+        return fail(PD_ERR_NOT_SPD, "a pivot of a factorised matrix was not positive");
     }
     return PD_OK;
     PD_API_END

@@ -174,7 +174,7 @@ struct AxBases {
     const float4* add;     // added to the result, or null
     float4* out;
     // of the launch (a batched one reads them from `single`, not from its slots):
-    bool once = false;     // the matrix leaves L2 first (see launch_products in k_dd.cu)
+    bool once = false;     // the matrix leaves L2 first (see product in k_dd.cu)
     bool late = false;     // the next kernel of the chain is not started before this one ends
 };
 struct AxDesc {
