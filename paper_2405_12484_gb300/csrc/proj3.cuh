@@ -391,7 +391,7 @@ static __device__ __forceinline__ void volume_targets(const float (&s)[3], float
 // condition number and C - I a rounding relative to 1; the other bounds are where these targets are as exact as the SVD's.
 // Root-mean-square errors of R, V and sigma / sigma_1 over 2,000 orientations in 2^-24, SVD / these: sigma = (1, 1, 1) 4.8
 // 5.1 8.9 / 0.7 0.5 0.7, (1.2, 0.6, 0.6) 1.1 1.6 1.3 / 1.0 0.8 0.7, (1, 0.5, 0.5) 1.6 1.7 1.5 / 1.0 0.9 1.0 (geometric mean
-// of the ratios over 125 inside 0.54, 0.32, 0.43); outside, (1.92, 0.8, 0.8) 1.2 2.5 1.5 / 1.3 0.9 1.2, (0.48, 0.438, 0.4)
+// of the ratios over 125 inside 0.54, 0.32, 0.42); outside, (1.92, 0.8, 0.8) 1.2 2.5 1.5 / 1.3 0.9 1.2, (0.48, 0.438, 0.4)
 // 1.5 2.0 2.6 / 0.9 1.0 6.3, (0.504, 0.21, 0.21) 1.6 2.1 1.9 / 7.6 6.4 3.6.  Everything else takes svd3 and
 // volume_targets.  About 300 instructions against 1,050.
 struct Strain {
